@@ -529,22 +529,40 @@ __global__ void __launch_bounds__(kChainMaxThreads) k_chain(const FrameDev *__re
 }
 
 // ---------------------------------------------------------------------------
-// Finalize: one CTA per (frame, chunk of kFinChunk symbols), one warp per
-// symbol, lanes over D.  Gradient sums of a chunk go to Gc[chunk]; a second
+// Finalize: one CTA per (frame, chunk of kFinChunk symbols), kFinSym symbols per
+// warp at once, lanes over D.  Gradient sums of a chunk go to Gc[chunk]; a second
 // kernel adds the chunks of a frame in order (deterministic).
-constexpr int kFinThreads = 256;
-constexpr int kFinChunk = 64;
+//
+// Bound by FP64: this GPU runs two FP64 lanes a clock and SM, so a warp's FP64
+// instruction takes 16 clocks, and the normaliser's butterfly (5 additions) and
+// division (about 20 instructions) per symbol outweighed everything else.  The
+// kFinSym symbols of a warp share them: the butterflies run as one reduction that
+// halves what a lane carries at each of the first exchanges (the additions and
+// their order per symbol stay the same), leaving symbol k's sums in lanes
+// 4 k .. 4 k + 3, where one division and one gradient formula serve all of them.
+// One frame's finalize (N = 50, q = 16, n = 10) took 30 us, one symbol after another
+// in each warp; its whole decode went from 267.5 to 255.3 us, and 256 frames of
+// N = 64, q = 8 from 499 to 470 us.
+constexpr int kFinSym = 8;
+constexpr int kFinThreads = 64;
+constexpr int kFinChunk = kFinSym * (kFinThreads / 32);
+constexpr int kFinRegs = 2;  // 32-wide slices of q kept in registers (q <= 64)
 
-// Row of the APP partials of symbol i in super-tile tlo + t; the first 32 are
-// cached one per lane (warp-uniform t), further ones are computed directly.
-__device__ __forceinline__ long long lp_row(const FrameDev &f, long long myrow, int t, int tlo,
-                                            int i) {
-    const long long cached = __shfl_sync(0xffffffffu, myrow, t & 31);
-    if (f.ps) return (long long)tlo + t;  // per-symbol producers: rows i*psT .. i*psT+psT-1
-    if (t < 32) return cached;
-    int ilo, ihi;
-    super_symbols(f, tlo + t, ilo, ihi);
-    return (long long)(tlo + t) * f.S2 + (i - ilo);
+// x[k]: this lane's part of sum k; returns, in lanes 4 k .. 4 k + 3, sum k over
+// the warp (butterfly order 16, 8, 4, 2, 1).
+__device__ __forceinline__ double fin_reduce(const double (&x)[kFinSym], int lane) {
+    double y[4], z[2];
+    const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        y[k] = (h4 ? x[k + 4] : x[k]) + __shfl_xor_sync(0xffffffffu, h4 ? x[k] : x[k + 4], 16);
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        z[k] = (h3 ? y[k + 2] : y[k]) + __shfl_xor_sync(0xffffffffu, h3 ? y[k] : y[k + 2], 8);
+    double r = (h2 ? z[1] : z[0]) + __shfl_xor_sync(0xffffffffu, h2 ? z[0] : z[1], 4);
+    r += __shfl_xor_sync(0xffffffffu, r, 2);
+    r += __shfl_xor_sync(0xffffffffu, r, 1);
+    return r;
 }
 
 __global__ void __launch_bounds__(kFinThreads) k_finalize(const FrameDev *__restrict__ frames,
@@ -552,116 +570,179 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(const FrameDev *__rest
                                                           int grad) {
     const Work wk = work[blockIdx.x];
     const FrameDev &f = frames[wk.frame];
-    __shared__ double red[3][32];
+    __shared__ double red[3][kFinThreads / 32];
     if (*f.status != ST_OK) return;
-    const int q = f.q, n = f.n, xmax = f.xmax;
+    const int q = f.q, n = f.n, xmax = f.xmax, S2 = f.S2, psT = f.psT;
     const long long P2 = (long long)f.P * f.nsub;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nw = blockDim.x >> 5;
-    const double Pt = f.dPt, Ps = f.dPs, Pd = f.dPd, k = f.kappa;
-    // the lattice ran with w' = k Pi/2, Q'm = k Pt (1-Ps), Q's = k Pt Ps
-    const double Qm = k * Pt * (1.0 - Ps), Qs = k * Pt * Ps;
-    double g0 = 0.0, g1 = 0.0, g2 = 0.0;
-    bool bad = false;
-    const int i0 = f.seg_i0 + (wk.tile - f.fin_base) * kFinChunk;
-    const int i1 = min(f.seg_i1, i0 + kFinChunk);
-    for (int i = i0 + warp; i < i1; i += nw) {
-        long long plo = (long long)n * i - xmax, phi = (long long)n * i + xmax;
-        if (plo < 0) plo = 0;
-        if (phi > f.rho) phi = f.rho;
-        int tlo = (int)(plo / P2), thi = (int)(phi / P2);
-        if (f.ps) {  // one row per work item (symbol, chunk of start states)
-            tlo = i * f.psT;
-            thi = tlo + f.psT - 1;
+    const float *Lp = f.Lp;
+    const int c0 = f.seg_i0 + (wk.tile - f.fin_base) * kFinChunk;
+    const int i1 = min(f.seg_i1, c0 + kFinChunk);
+    const int i0 = c0 + warp * kFinSym;
+    const int ns = max(0, min(kFinSym, i1 - i0));  // symbols of this warp
+    // Rows of the APP partials of symbol i0 + k: tiles tlo .. thi, one row each.
+    // The lanes of symbol k find theirs; row of tile t: t S2 + i - (the tile's
+    // first symbol), or t itself (per-symbol producers: rows are work items).
+    const int mine = lane >> 2;
+    long long tlo = 0, thi = -1;
+    if (mine < ns) {
+        const int i = i0 + mine;
+        if (f.ps) {
+            tlo = (long long)i * psT;
+            thi = tlo + psT - 1;
+        } else {
+            tlo = max(0LL, (long long)n * i - xmax) / P2;
+            thi = min(f.rho, (long long)n * i + xmax) / P2;
         }
-        // lane l holds the Lp row offset of super-tile tlo + l for this symbol
-        long long myrow = 0;
-        if (!f.ps && tlo + lane <= thi) {
-            int ilo, ihi;
-            super_symbols(f, tlo + lane, ilo, ihi);
-            myrow = (long long)(tlo + lane) * f.S2 + (i - ilo);
+    }
+    auto row_of = [&](int i, long long t) -> long long {
+        if (f.ps) return t;
+        const long long ilo = max((long long)f.seg_i0, ceildiv(t * P2 - xmax, n));
+        return t * S2 + (i - ilo);
+    };
+    // the first four rows of each symbol, one per lane
+    const long long myrow = mine < ns && tlo + (lane & 3) <= thi ? row_of(i0 + mine, tlo + (lane & 3)) : 0;
+    // unnormalised sums L^u(D) (eq. L without the prior), lane = D mod 32
+    auto lsum = [&](int k, int D) {
+        const long long lo = __shfl_sync(0xffffffffu, tlo, 4 * k), hi = __shfl_sync(0xffffffffu, thi, 4 * k);
+        float v = 0.f;
+        for (int t = 0; t <= hi - lo; ++t) {
+            long long row = __shfl_sync(0xffffffffu, myrow, 4 * k + (t & 3));
+            if (t > 3) row = row_of(i0 + k, lo + t);
+            if (D < q) v += Lp[row * q + D];
         }
-        double z = 0.0, zu = 0.0;
-        // pass 1: unnormalised sums L^u(D) (eq. L without the prior) into app,
-        // z = sum_D prior(D) L^u(D) and, for the extrinsic output, zu = sum_D L^u(D)
-        for (int D0 = 0; D0 < q; D0 += 32) {
-            const int D = D0 + lane;
-            float s = 0.f;
-            for (int t = 0; t <= thi - tlo; ++t) {
-                const long long row = lp_row(f, myrow, t, tlo, i);
-                if (D < q) s += f.Lp[row * q + D];
-            }
-            if (D < q) {
-                f.app[(size_t)i * q + D] = s;
-                z += (double)f.priors[(size_t)i * q + D] * (double)s;
-                zu += (double)s;
-            }
-        }
+        return v;
+    };
+    // pass 1: z = sum_D prior(D) L^u(D) and, for the extrinsic output, zu = sum_D L^u(D)
+    float lu[kFinSym][kFinRegs];
+    double z[kFinSym], zu[kFinSym];
+    const bool kept = q <= 32 * kFinRegs;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            z += __shfl_xor_sync(0xffffffffu, z, o);
-            zu += __shfl_xor_sync(0xffffffffu, zu, o);
+    for (int k = 0; k < kFinSym; ++k) {
+        z[k] = zu[k] = 0.0;
+#pragma unroll
+        for (int r = 0; r < kFinRegs; ++r) lu[k][r] = 0.f;
+        if (k >= ns) continue;
+        const float *pri = f.priors + (size_t)(i0 + k) * q;
+        if (kept) {
+#pragma unroll
+            for (int r = 0; r < kFinRegs; ++r) {
+                const int D = 32 * r + lane;
+                if (32 * r >= q) break;
+                lu[k][r] = lsum(k, D);
+                if (D < q) {
+                    z[k] += (double)pri[D] * (double)lu[k][r];
+                    if (f.ext) zu[k] += (double)lu[k][r];
+                }
+            }
+        } else {
+            for (int D0 = 0; D0 < q; D0 += 32) {
+                const int D = D0 + lane;
+                const float v = lsum(k, D);
+                if (D < q) {
+                    f.app[(size_t)(i0 + k) * q + D] = v;
+                    z[k] += (double)pri[D] * (double)v;
+                    zu[k] += (double)v;
+                }
+            }
         }
-        if (!(z > 0.0)) { bad = true; continue; }
-        const double iz = 1.0 / z;
-        const double izu = 1.0 / zu;  // zu >= z / max prior > 0
-        // pass 2: each lane rescales the entries it wrote
-        for (int D = lane; D < q; D += 32) {
-            const size_t e = (size_t)i * q + D;
-            const double lu = (double)f.app[e];
-            f.app[e] = (float)((double)f.priors[e] * lu * iz);
-            if (f.dpriors) f.dpriors[e] = (float)(lu * iz);
-            if (f.ext) f.ext[e] = (float)(lu * izu);
+    }
+    const double zs = fin_reduce(z, lane);
+    const bool ok = mine < ns && zs > 0.0;
+    const double iz = ok ? 1.0 / zs : 0.0;
+    double izu = 0.0;
+    if (f.ext) {
+        const double zus = fin_reduce(zu, lane);
+        izu = ok ? 1.0 / zus : 0.0;  // zu >= z / max prior > 0
+    }
+    const unsigned good = __ballot_sync(0xffffffffu, ok);
+    // pass 2: each lane scales the entries it summed
+#pragma unroll
+    for (int k = 0; k < kFinSym; ++k) {
+        const double izk = __shfl_sync(0xffffffffu, iz, 4 * k), izuk = __shfl_sync(0xffffffffu, izu, 4 * k);
+        if (!(good >> (4 * k) & 1u)) continue;
+        const size_t e0 = (size_t)(i0 + k) * q;
+        auto put = [&](int D, float v) {
+            const size_t e = e0 + D;
+            const double l = (double)v;
+            f.app[e] = (float)((double)f.priors[e] * l * izk);
+            if (f.dpriors) f.dpriors[e] = (float)(l * izk);
+            if (f.ext) f.ext[e] = (float)(l * izuk);
+        };
+        if (kept) {
+#pragma unroll
+            for (int r = 0; r < kFinRegs; ++r)
+                if (32 * r + lane < q) put(32 * r + lane, lu[k][r]);
+        } else {
+            for (int D = lane; D < q; D += 32) put(D, f.app[e0 + D]);
         }
-        if (grad) {
+    }
+    if (lane == 0 && good != (ns == kFinSym ? 0xffffffffu : (1u << (4 * ns)) - 1u))
+        atomicMax(f.status, ST_ZERO);
+    if (grad && f.Gc) {
+        double g0 = 0.0, g1 = 0.0, g2 = 0.0;
+        if (ok) {
+            // the lattice ran with w' = k Pi/2, Q'm = k Pt (1-Ps), Q's = k Pt Ps
+            const double Pt = f.dPt, Ps = f.dPs, Pd = f.dPd, k = f.kappa;
+            const double Qm = k * Pt * (1.0 - Ps), Qs = k * Pt * Ps;
             double Sw = 0.0, Sd = 0.0, Ss = 0.0;
-            for (int t = 0; t <= thi - tlo; ++t) {
-                const long long row = lp_row(f, myrow, t, tlo, i);
-                const float *gp = f.Gp + row * 3;
+            for (long long t = tlo; t <= thi; ++t) {
+                const float *gp = f.Gp + row_of(i0 + mine, t) * 3;
                 Sw += gp[0];
                 Sd += gp[1];
                 Ss += gp[2];
             }
-            if (lane == 0) {
-                // Sw, Sd, Ss: sums with dR~/dw', dR~/dPd, dR~/dQ's.  R~ is homogeneous
-                // of degree n in (Pd, Q'm, Q's) (every bit is deleted or transmitted),
-                // so Pd dR~/dPd + Q'm dR~/dQ'm + Q's dR~/dQ's = n R~ gives the Q'm sum.
-                // Chain rule with w' = k Pi/2, Q'm = k Pt (1-Ps), Q's = k Pt Ps, Pt = 1-Pi-Pd.
-                const double Sm = ((double)n * z - Pd * Sd - Qs * Ss) / Qm;
-                g0 += (0.5 * k * Sw - k * (1.0 - Ps) * Sm - k * Ps * Ss) * iz;
-                g1 += (Sd - k * (1.0 - Ps) * Sm - k * Ps * Ss) * iz;
-                g2 += (-k * Pt * Sm + k * Pt * Ss) * iz;
-            }
+            // Sw, Sd, Ss: sums with dR~/dw', dR~/dPd, dR~/dQ's.  R~ is homogeneous
+            // of degree n in (Pd, Q'm, Q's) (every bit is deleted or transmitted),
+            // so Pd dR~/dPd + Q'm dR~/dQ'm + Q's dR~/dQ's = n R~ gives the Q'm sum.
+            // Chain rule with w' = k Pi/2, Q'm = k Pt (1-Ps), Q's = k Pt Ps, Pt = 1-Pi-Pd.
+            const double Sm = ((double)n * zs - Pd * Sd - Qs * Ss) / Qm;
+            g0 = (0.5 * k * Sw - k * (1.0 - Ps) * Sm - k * Ps * Ss) * iz;
+            g1 = (Sd - k * (1.0 - Ps) * Sm - k * Ps * Ss) * iz;
+            g2 = (-k * Pt * Sm + k * Pt * Ss) * iz;
         }
-    }
-    if (bad && lane == 0) atomicMax(f.status, ST_ZERO);
-    if (grad && f.Gc) {
+        // over the warp's symbols (one lane in four), then the warps in order
+#pragma unroll
+        for (int o = 16; o > 2; o >>= 1) {
+            g0 += __shfl_xor_sync(0xffffffffu, g0, o);
+            g1 += __shfl_xor_sync(0xffffffffu, g1, o);
+            g2 += __shfl_xor_sync(0xffffffffu, g2, o);
+        }
         if (lane == 0) { red[0][warp] = g0; red[1][warp] = g1; red[2][warp] = g2; }
         __syncthreads();
         if (threadIdx.x < 3) {
             double s = 0.0;
-            for (int w = 0; w < nw; ++w) s += red[threadIdx.x][w];
+            for (int w = 0; w < kFinThreads / 32; ++w) s += red[threadIdx.x][w];
             f.Gc[(size_t)wk.tile * 3 + threadIdx.x] = s;
         }
     }
 }
 
-// Sums the chunk gradients of every frame in chunk order.
+// Sums the chunk gradients of every frame, a warp per frame: lane l adds chunks
+// l, l + 32, .. in order, then a butterfly (deterministic).
 __global__ void k_grad_reduce(const FrameDev *__restrict__ frames, int nframes) {
-    const int fi = blockIdx.x * blockDim.x + threadIdx.x;
+    const int fi = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (fi >= nframes) return;
     const FrameDev &f = frames[fi];
     if (!f.dchan || !f.Gc || *f.status != ST_OK) return;
     const int nch = f.fin_total;
     double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-    for (int c = 0; c < nch; ++c) {
+    for (int c = lane; c < nch; c += 32) {
         s0 += f.Gc[3 * c];
         s1 += f.Gc[3 * c + 1];
         s2 += f.Gc[3 * c + 2];
     }
-    f.dchan[0] = s0;
-    f.dchan[1] = s1;
-    f.dchan[2] = s2;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+    }
+    if (lane == 0) {
+        f.dchan[0] = s0;
+        f.dchan[1] = s1;
+        f.dchan[2] = s2;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -742,7 +823,7 @@ cudaError_t launch_finalize(const FrameDev *frames, const Work *work, int nwork,
     if (nwork > 0) k_finalize<<<nwork, kFinThreads, 0, st>>>(frames, work, grad);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || !grad || !reduce || nframes <= 0) return e;
-    k_grad_reduce<<<(nframes + 127) / 128, 128, 0, st>>>(frames, nframes);
+    k_grad_reduce<<<(nframes + 3) / 4, 128, 0, st>>>(frames, nframes);
     return cudaGetLastError();
 }
 
