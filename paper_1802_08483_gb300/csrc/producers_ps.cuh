@@ -46,6 +46,40 @@ __device__ __forceinline__ void eval_metric_x(const FrameDev &f, long long p, ui
     }
 }
 
+// Sums acc[j] over the G lanes of a group (butterfly order G/2, .., 1) and stores
+// row[j], j < MN.  Every exchange halves the values a lane carries (lane gl ends
+// with values gl V / G ..): about MN shuffles and additions in all where a
+// butterfly per value took MN log2 G of each, and neighbouring lanes store
+// neighbouring values.  The additions and their order per value are the same.
+// 16 frames (N = 1000, q = 16, n = 10, I = 2, xmax = 85): the whole decode 9.74 ms
+// with a butterfly per value, 6.25 ms with this; bound by the lattices since.
+template <int MNC, int G>
+__device__ __forceinline__ void ps_reduce_store(const float (&acc)[MNC], int gl, int MN, bool store,
+                                                float *row) {
+    constexpr int V = MNC <= G ? G : (MNC + G - 1) / G * G;  // values, padded with zeros
+    float x[V];
+#pragma unroll
+    for (int j = 0; j < V; ++j) x[j] = j < MNC ? acc[j < MNC ? j : 0] : 0.f;
+#pragma unroll
+    for (int o = G / 2, w = V / 2; o > 0; o >>= 1, w >>= 1) {
+        const bool up = (gl & o) != 0;
+#pragma unroll
+        for (int j = 0; j < V / 2; ++j) {
+            if (j < w) {
+                const float keep = up ? x[j + w] : x[j], give = up ? x[j] : x[j + w];
+                x[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+            }
+        }
+    }
+    if (store) {
+#pragma unroll
+        for (int t = 0; t < V / G; ++t) {
+            const int j = gl * (V / G) + t;
+            if (j < MN) row[j] = x[t];
+        }
+    }
+}
+
 template <int NB, int IB>
 __global__ void __launch_bounds__(kThreads) k_fwd_ps(const FrameDev *__restrict__ frames,
                                                      const Work *__restrict__ work) {
@@ -81,17 +115,13 @@ __global__ void __launch_bounds__(kThreads) k_fwd_ps(const FrameDev *__restrict_
                     if (j < MN) acc[j] = fmaf(w, v[j], acc[j]);
             }
         }
-#pragma unroll
-        for (int j = 0; j < MNC; ++j) {
-            if (j < MN) {
-                for (int o = G >> 1; o > 0; o >>= 1)
-                    acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
-            }
-        }
-        if (valid && gl == 0) {
-#pragma unroll
-            for (int j = 0; j < MNC; ++j)
-                if (j < MN) Wi[(size_t)s * f.MNS + j] = acc[j];
+        float *Ws = Wi + (size_t)s * f.MNS;
+        switch (G) {
+            case 32: ps_reduce_store<MNC, 32>(acc, gl, MN, valid, Ws); break;
+            case 16: ps_reduce_store<MNC, 16>(acc, gl, MN, valid, Ws); break;
+            case 8: ps_reduce_store<MNC, 8>(acc, gl, MN, valid, Ws); break;
+            case 4: ps_reduce_store<MNC, 4>(acc, gl, MN, valid, Ws); break;
+            default: ps_reduce_store<MNC, 2>(acc, gl, MN, valid, Ws);
         }
     }
 }
