@@ -7,7 +7,7 @@ namespace mdk {
 cudaError_t launch_fwd_I1(int n, const FrameDev *frames, const Work *work, int nwork, size_t smem,
                           cudaStream_t st) {
     switch (n) {
-        MAPDEC_FOR_N(MAPDEC_CASE_FWD)
+        MAPDEC_FOR_N_LONG(MAPDEC_CASE_FWD)
         default: return cudaErrorNotSupported;
     }
 }
@@ -22,7 +22,7 @@ cudaError_t launch_fwd_tc_I1(int n, const FrameDev *frames, const Work *work, in
 
 cudaError_t launch_rmetric_I1(int n, const FrameDev *frame, long long nthreads, cudaStream_t st) {
     switch (n) {
-        MAPDEC_FOR_N(MAPDEC_CASE_RM)
+        MAPDEC_FOR_N_LONG(MAPDEC_CASE_RM)
         default: return cudaErrorNotSupported;
     }
 }

@@ -8,7 +8,7 @@ cudaError_t launch_bwd_I3_plain(int n, const FrameDev *frames, const Work *work,
                                   size_t smem, cudaStream_t st) {
     const bool grad = false;
     switch (n) {
-        MAPDEC_FOR_N(MAPDEC_CASE_BWDX)
+        MAPDEC_FOR_N_LONG(MAPDEC_CASE_BWDX)
         default: return cudaErrorNotSupported;
     }
 }

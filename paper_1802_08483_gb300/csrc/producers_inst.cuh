@@ -93,7 +93,7 @@ cudaError_t launch_rmetric_t(const FrameDev *fr, long long nthreads, cudaStream_
 
 }  // namespace mdk
 
-// Per-I dispatch over n = 1..12.
+// Per-I dispatch over n = 1..12 (to 15 where said).
 #define MAPDEC_CASE_FWD(NV) case NV: return launch_fwd_t<NV, MAPDEC_IB>(frames, work, nwork, smem, st);
 #define MAPDEC_CASE_BWD(NV)                                                            \
     case NV:                                                                           \
@@ -108,4 +108,6 @@ cudaError_t launch_rmetric_t(const FrameDev *fr, long long nthreads, cudaStream_
 #define MAPDEC_CASE_FWDPS(NV) case NV: return launch_fwd_ps_t<NV, MAPDEC_IB>(frames, work, nwork, st);
 #define MAPDEC_CASE_BWDPS(NV) case NV: return launch_bwd_ps_t<NV, MAPDEC_IB, grad>(frames, work, nwork, smem, st);
 #define MAPDEC_FOR_N_TC(M) M(4) M(5) M(6) M(7) M(8) M(9) M(10) M(11) M(12)
+// Decode-mode producers and the receiver metric of one codebook go on to n = 15.
+#define MAPDEC_FOR_N_LONG(M) MAPDEC_FOR_N(M) M(13) M(14) M(15)
 #define MAPDEC_FOR_N(M) M(1) M(2) M(3) M(4) M(5) M(6) M(7) M(8) M(9) M(10) M(11) M(12)

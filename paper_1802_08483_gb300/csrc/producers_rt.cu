@@ -36,7 +36,9 @@ size_t bwd_smem_bytes(const FrameDev &f, bool grad) {
     return 4 * fl;
 }
 
-bool specialised(int n, int I) { return n >= 1 && n <= kMaxSpecN && I >= 1 && I <= 3; }
+bool specialised(int n, int I, bool decode) {
+    return n >= 1 && n <= (decode ? kMaxSpecDecodeN : kMaxSpecN) && I >= 1 && I <= 3;
+}
 
 // ---------------------------------------------------------------------------
 // Priors of a frame as the B operand of the W contraction: three bf16 pieces,
@@ -165,7 +167,7 @@ cudaError_t launch_fwd_tc(int n, int I, const FrameDev *frames, const Work *work
 
 cudaError_t launch_fwd(int n, int I, const FrameDev *frames, const Work *work, int nwork,
                        size_t smem, cudaStream_t st) {
-    if (specialised(n, I)) {
+    if (specialised(n, I, true)) {
         if (I == 1) return launch_fwd_I1(n, frames, work, nwork, smem, st);
         if (I == 2) return launch_fwd_I2(n, frames, work, nwork, smem, st);
         return launch_fwd_I3(n, frames, work, nwork, smem, st);
@@ -175,7 +177,7 @@ cudaError_t launch_fwd(int n, int I, const FrameDev *frames, const Work *work, i
 
 cudaError_t launch_bwd(int n, int I, bool grad, const FrameDev *frames, const Work *work,
                        int nwork, size_t smem, cudaStream_t st) {
-    if (specialised(n, I)) {
+    if (specialised(n, I, !grad)) {
         if (I == 1) return launch_bwd_I1(n, grad, frames, work, nwork, smem, st);
         if (I == 2) return launch_bwd_I2(n, grad, frames, work, nwork, smem, st);
         return launch_bwd_I3(n, grad, frames, work, nwork, smem, st);
@@ -185,7 +187,7 @@ cudaError_t launch_bwd(int n, int I, bool grad, const FrameDev *frames, const Wo
 
 cudaError_t launch_rmetric(int n, int I, const FrameDev *frame, long long nthreads,
                            cudaStream_t st) {
-    if (specialised(n, I)) {
+    if (specialised(n, I, true)) {
         if (I == 1) return launch_rmetric_I1(n, frame, nthreads, st);
         if (I == 2) return launch_rmetric_I2(n, frame, nthreads, st);
         return launch_rmetric_I3(n, frame, nthreads, st);
