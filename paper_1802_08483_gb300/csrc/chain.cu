@@ -597,8 +597,9 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(const FrameDev *__rest
     }
     auto row_of = [&](int i, long long t) -> long long {
         if (f.ps) return t;
-        const long long ilo = max((long long)f.seg_i0, ceildiv(t * P2 - xmax, n));
-        return t * S2 + (i - ilo);
+        // i - ceil((t P2 - xmax) / n), the tile's first symbol not before the segment's
+        const unsigned past = (unsigned)((long long)n * i - t * P2 + xmax) / (unsigned)n;
+        return t * S2 + min(i - f.seg_i0, (int)past);
     };
     // the first four rows of each symbol, one per lane
     const long long myrow = mine < ns && tlo + (lane & 3) <= thi ? row_of(i0 + mine, tlo + (lane & 3)) : 0;
@@ -606,10 +607,16 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(const FrameDev *__rest
     auto lsum = [&](int k, int D) {
         const long long lo = __shfl_sync(0xffffffffu, tlo, 4 * k), hi = __shfl_sync(0xffffffffu, thi, 4 * k);
         float v = 0.f;
-        for (int t = 0; t <= hi - lo; ++t) {
-            long long row = __shfl_sync(0xffffffffu, myrow, 4 * k + (t & 3));
-            if (t > 3) row = row_of(i0 + k, lo + t);
-            if (D < q) v += Lp[row * q + D];
+        for (int t0 = 0; t0 <= hi - lo; t0 += 32) {
+            // up to four rows from the start, more found a warp's width at a time
+            long long r = myrow;
+            const bool wide = hi - lo > 3;
+            if (wide) r = lo + t0 + lane <= hi ? row_of(i0 + k, lo + t0 + lane) : 0;
+            const int cnt = (int)min(32LL, hi - lo + 1 - t0);
+            for (int t = 0; t < cnt; ++t) {
+                const long long row = __shfl_sync(0xffffffffu, r, wide ? t : 4 * k + t);
+                if (D < q) v += Lp[row * q + D];
+            }
         }
         return v;
     };

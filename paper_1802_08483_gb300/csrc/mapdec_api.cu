@@ -204,6 +204,7 @@ struct FrameHost {
     bool store = false;     // keep the receiver metrics in HBM for the APP producer
     bool tc = false;        // forward producer on the tensor cores
     bool tcb = false;       // APP producer on the tensor cores
+    bool split = false;     // APP super-tiles may be shortened to fill the GPU
     std::vector<float> phi0, phiN;  // boundary drift priors (stream decoding), or empty
     int64_t phi_off = 0;    // float offset of phi0 (then phiN) in the batch's buffer
 };
@@ -463,6 +464,32 @@ size_t frame_scratch_floats_seg(const FrameDev &f, int K, int S, bool grad) {
     return s;
 }
 
+// APP super-tiles short enough for a launch to fill the GPU.  plan_shape's
+// super-tiles of 256 positions amortise a CTA's set-up over a large batch, but a
+// single frame or a checkpointed batch's segment is then a handful of CTAs on 152
+// SMs: halve them while the launch (ctas CTAs with the present ones) has fewer
+// than two per SM.  Decode mode only: the APP sums' order over positions follows
+// the super-tiles, and gradients keep theirs.
+// Whole decodes before and after: one frame N=50 q=16 255 -> 196 us, N=300 q=32
+// 712 -> 638 us; 8 frames N=8000 q=64, checkpointed, 411 -> 287 ms.
+int supertile_split(long long ctas) {
+    const int sms = device_sms() > 0 ? device_sms() : 152;
+    int d = 1;
+    while (d < 256 && ctas * d < 2LL * sms) d *= 2;
+    return d;
+}
+// A frame's super-tiles at its largest received length (tau + xmax), so that a
+// handle planned for it and a frame planned for its own length agree.
+int most_supertiles(const FrameDev &f) {
+    const long long P2 = (long long)f.P * f.nsub;
+    return (int)(((long long)f.n * f.N + f.xmax + P2) / P2);
+}
+void split_supertiles(FrameDev &f, int d) {
+    f.nsub = std::max(1, f.nsub / d);
+    f.S2 = (int)(((long long)f.P * f.nsub - 1 + 2LL * f.xmax) / f.n + 2);
+    f.T2 = (f.T + f.nsub - 1) / f.nsub;
+}
+
 double frame_cost(const FrameDev &f) {
     // algorithmic flop estimate used for load balancing and reporting
     const double cells = (f.I + 1) * f.n * (f.n + 1) / 2.0 + (f.n + 1);
@@ -694,7 +721,9 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
     b->nframes = nf;
     b->flags = flags;
     b->grad = (flags & MAPDEC_BATCH_GRAD) != 0;
+    b->segmented = (flags & MAPDEC_BATCH_SEGMENTED) != 0;
     b->fr.resize(nf);
+    std::map<std::pair<int, int>, long long> class_ctas;  // APP-producer CTAs per (n, I) launch
     for (int i = 0; i < nf; ++i) {
         FrameHost &h = b->fr[i];
         h.d = frames[i];
@@ -817,11 +846,12 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
             K = std::max(1, std::min(K, h.d.N));
             h.segK = K;
             h.nseg = (h.d.N + K - 1) / K;
-            h.scratch_floats = frame_scratch_floats_seg(h.dev, K, h.nseg, b->grad);
-        } else {
-            h.scratch_floats = frame_scratch_floats(h.dev, b->grad);
-            if (h.store) h.scratch_floats += rup(metric_store_floats(h.dev), 64);
         }
+        h.split = !b->grad && !per_sym && !h.tcb && !(tuned && tu.nsub > 0) &&
+                  !std::getenv("MAPDEC_FORCE_NSUB");
+        if (h.split)
+            class_ctas[{h.d.n, h.d.I}] += b->segmented ? seg_supertiles(h.dev, h.segK) - 2
+                                                       : most_supertiles(h.dev);
         h.cost = frame_cost(h.dev);
         h.rx_off = b->rx_total;
         b->rx_total += h.d.rx_len;  // dense: the caller's concatenation, one copy
@@ -833,6 +863,15 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
         b->cw_total += (int64_t)h.cw.size();
         h.phi_off = b->phi_total;
         b->phi_total += (int64_t)(h.phi0.size() + h.phiN.size());
+    }
+    for (auto &h : b->fr) {
+        if (h.split) split_supertiles(h.dev, supertile_split(class_ctas[{h.d.n, h.d.I}]));
+        if (b->segmented) {
+            h.scratch_floats = frame_scratch_floats_seg(h.dev, h.segK, h.nseg, b->grad);
+        } else {
+            h.scratch_floats = frame_scratch_floats(h.dev, b->grad);
+            if (h.store) h.scratch_floats += rup(metric_store_floats(h.dev), 64);
+        }
     }
     // resident buffers
     b->d_rx = (uint8_t *)b->dalloc(b->rx_total + 64);
@@ -895,8 +934,7 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
     b->region_floats = rup(b->scratch_floats, 64);
     b->d_scratch = (float *)b->dalloc(b->region_floats * 4 * b->regions + 256);
     // per-wave descriptors and work tables
-    const bool segmented = (flags & MAPDEC_BATCH_SEGMENTED) != 0;
-    b->segmented = segmented;
+    const bool segmented = b->segmented;
     if (const char *e = std::getenv("MAPDEC_CHAIN_THREADS")) b->chain_threads = std::atoi(e);  // A/B override
     for (size_t wi = 0; wi < b->waves.size(); ++wi) {
         Wave &w = b->waves[wi];
@@ -1868,6 +1906,7 @@ int mapdec_decode_noalloc(const mapdec_frame_desc_t *frame, const uint8_t *rx_de
 
     FrameDev f{};
     plan_shape(f, d, false, 0);
+    split_supertiles(f, supertile_split(most_supertiles(f)));
     // carve the arena (every region 256-byte aligned)
     size_t off = 0;
     auto take = [&](size_t bytes) -> size_t {

@@ -46,6 +46,39 @@ def test_finalize_edges(N, q, n):
                                             priors=fr.priors)[1])
 
 
+# compiled lattices of long codewords, and run-time ones past them
+@pytest.mark.parametrize("n,I", [(13, 1), (14, 1), (15, 1), (13, 2), (15, 2), (13, 3), (14, 3),
+                                 (15, 3), (16, 2), (20, 1)])
+def test_long_codewords(n, I):
+    N, q, xmax = 14, 6, 18
+    fr = synth.make_frame(np.random.default_rng(n * I), q, n, N, I, xmax, 0.03, 0.03, 0.01,
+                          dirichlet=True)
+    ref, ll_ref = oracle.decode(fr.codebook, N, 0.03, 0.03, 0.01, I, xmax, fr.rx,
+                                priors=fr.priors, kappa=2.0)
+    b = mapdec.Batch([fr], flags=mapdec.MAPDEC_BATCH_GRAPH)
+    st, app, ll = b.decode(fr.rx, fr.priors.reshape(-1))
+    b.close()
+    assert st == 0
+    check_app(app.reshape(N, q), ref)
+    check_ll(ll[0], ll_ref)
+
+
+def test_many_supertiles_per_symbol():
+    """A lone frame's super-tiles are short: a symbol's window spans more than the
+    32 partial rows that finalize looks up at a time."""
+    N, q, n, I, xmax = 30, 64, 6, 3, 230
+    fr = synth.make_frame(np.random.default_rng(5), q, n, N, I, xmax, 0.05, 0.05, 0.01,
+                          dirichlet=True)
+    ref, ll_ref = oracle.decode(fr.codebook, N, 0.05, 0.05, 0.01, I, xmax, fr.rx,
+                                priors=fr.priors, kappa=2.0)
+    b = mapdec.Batch([fr], flags=mapdec.MAPDEC_BATCH_GRAPH)
+    st, app, ll = b.decode(fr.rx, fr.priors.reshape(-1))
+    b.close()
+    assert st == 0
+    check_app(app.reshape(N, q), ref)
+    check_ll(ll[0], ll_ref)
+
+
 # lanes per group 2, 2, 4, 8, 16, 32, 32; lengths below, at and above the group's lanes
 @pytest.mark.parametrize("q,n,I", [(2, 4, 1), (3, 3, 2), (5, 5, 2), (9, 4, 3), (17, 5, 3),
                                    (33, 6, 1), (40, 12, 3)])
