@@ -367,9 +367,11 @@ typedef struct {
                             the APP producer on the CUDA cores); 1: both producers on
                             the tensor cores wherever the class supports them (see
                             mapdec_batch_tc_frames); 2: FP32 CUDA-core producers */
-    int chain_threads;   /* block size of the recursion kernel: 128, 256 or 512
-                            (0 = 256); the batch takes the value of its last frame
-                            whose class sets it */
+    int chain_threads;   /* block size of the recursion kernel of batches with more
+                            recursions (two per frame) than SMs, or several waves:
+                            128, 256 or 512 (0 = 256); the batch takes the value of
+                            its last frame whose class sets it.  Smaller launches
+                            size their recursions by the frames' states */
 } mapdec_tune_t;
 
 /* Set (t != NULL) or remove (t == NULL) the entry of class (q, n, I). */

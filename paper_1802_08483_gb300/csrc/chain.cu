@@ -1,23 +1,14 @@
 // Sequential parts of the decoder and small helper kernels.
 //
 //   k_pack     : received bits (one per byte) -> 32-bit words.
-//   k_chain    : the forward recursion (eqs. alpha_prenorm, alpha_norm) or the
-//                backward recursion (eq. beta, normalised by its sum) of one
-//                frame, one CTA per (frame, direction).  The per-symbol
-//                transition sums W_i(s', j) stream from global memory into
-//                shared memory by 1-D bulk copies (cp.async.bulk) completed on
-//                mbarriers, double-buffered, while the previous chunk is used.
-//                Rows are kept exponentially tilted (see below) so that FP32
-//                holds them; the forward chain keeps the exact FP64 record of
-//                every normaliser and tilt and writes log P(Y).
+//   k_chain    : the recursions (chain_kern.cuh), dispatched here.
 //   k_finalize : APPs (eq. L, normalised over D), extrinsic outputs (eq. L
 //                without the symbol's own prior), d logP / d prior and the
 //                FP64 reduction of the channel-parameter gradient
 //                (k_grad_reduce adds the chunks of a frame in order).
 #include <cstdlib>
 
-#include "mapdec_dev.cuh"
-#include "mapdec_kernels.h"
+#include "chain_kern.cuh"
 
 namespace mdk {
 
@@ -43,9 +34,15 @@ __global__ void k_pack(const FrameDev *__restrict__ frames, const uint8_t *const
 }
 
 // ---------------------------------------------------------------------------
-constexpr int kChainMaxThreads = 512;
-constexpr int kChainThreads = 256;  // default block size
-constexpr int kMaxStages = 8;
+// The recursions of launches with more of them than SMs (k_chain_crowd).  The same
+// recursion and the same sums in the same order as k_chain, one CTA per (frame,
+// direction), with a few registers and as little shared memory as two staged
+// chunks take, so that several share an SM with each other and with the producers
+// of other waves; k_chain's lower latency needs an SM to itself (256 frames N = 64,
+// q = 8: 470 us a decode with this kernel, 520 to 590 with k_chain at two and
+// three CTAs per SM; 512 mixed frames in waves of 64: 167 ms against 209 to 255).
+constexpr int kCrowdThreads = 256;  // default block size
+constexpr int kCrowdMaxThreads = 512;
 
 // Two FP32 sums at once (row sum and first moment); every thread gets the
 // same result (the warps' partials are added in one fixed order).
@@ -66,18 +63,11 @@ __device__ __forceinline__ void block_sum2(float a, float b, float &sa, float &s
     sb = y;
 }
 
-// Tilt controller (see k_chain).
-constexpr float kTiltGainMin = 0.02f;  // long-run smoothing of the entropy-rate estimate
-constexpr float kTiltStepMax = 0.02f;  // largest change of the tilt between two rows
-constexpr float kTiltMin = 0.2f, kTiltMax = 1.6f;
-constexpr int kTiltEvery = 4;    // steps between tilt updates once settled
-constexpr int kTiltSettle = 64;  // updates every step for the first steps
-
 // Geometry of chunk k of a step: the same for every symbol, relative to the
 // symbol's block of W (blocks are 16-byte aligned, so the aligned copy start,
 // the shift to row r0 and the copy size do not depend on the symbol).
 constexpr int kMaxChunks = 64;
-struct ChunkTab {
+struct CrowdTab {
     int d0[kMaxChunks], d1[kMaxChunks];  // owned states (alpha: destinations, beta: sources)
     int r0[kMaxChunks], r1[kMaxChunks];  // W rows staged
     int shift[kMaxChunks];               // floats between the aligned copy start and row r0
@@ -85,8 +75,8 @@ struct ChunkTab {
     uint32_t bytes[kMaxChunks];          // copy size
 };
 
-__device__ __forceinline__ void chunk_geom(const FrameDev &f, int dir, int k, ChunkTab &t) {
-    const int CD = f.chainCD, M = f.M;
+__device__ __forceinline__ void crowd_geom(const FrameDev &f, int dir, int k, CrowdTab &t) {
+    const int CD = f.crowdCD, M = f.M;
     const int d0 = k * CD, d1 = min(M, d0 + CD);
     int r0, r1;
     if (dir == 0) {  // destination s gets sources s - nI .. s + n
@@ -107,39 +97,16 @@ __device__ __forceinline__ void chunk_geom(const FrameDev &f, int dir, int k, Ch
     t.bytes[k] = a1 > a0 ? (uint32_t)(a1 - a0) * 4u : 16u;
 }
 
-// Exponential tilt.  The forward metric alpha_i(m) is the joint probability of
-// a received prefix of L = n i + m bits, so a row falls off roughly like
-// 2^{-h L} (h: entropy rate of the received bits) on top of the drift
-// posterior; the backward metric rises the same way.  Far apart in FP32, the
-// entries that carry the posterior would underflow.  The chains therefore store
-//   alpha^_i(m) = alpha_i(m) 2^{theta_i L} / Z_i,   beta^_i(m) = beta_i(m) 2^{-theta'_i L} / Y_i
-// with tilts theta driven toward h by the row sums: with a tilt theta a step
-// grows the row sum by about 2^{(theta - h) n}, so theta_{i+1} = theta_i -
-// g log2(growth) / n (g = 1/(steps+1), floored at kTiltGainMin); after the
-// first kTiltSettle steps it is updated every kTiltEvery steps from the mean
-// growth of the steps since.  The producers already weight every received bit
-// by 2 (theta = 1), so a step multiplies the transition sums by
-// 2^{(theta - 1) j} (j = received length) and pre-scales the source row by
-// 2^{(theta_{i+1} - theta_i)(m - mean)}.  Each new row is divided by the
-// power of two 2^e just below its sum c (exact; the row then sums to [1, 2)),
-// so Z_i is a power of two times the tilt factors, kept exactly in FP64, and
-// log P(Y) = log alpha^_N(rho - tau) + log Z_N - theta_N rho log 2.  The APP
-// producer applies the matching exact factor; the per-row constants cancel in
-// the APPs and in the gradient.
-//
-// The W rows of a step stream into shared memory in chunks of chainCD states
-// (plus the band halo in the forward direction) by 1-D bulk copies completed
-// on mbarriers, chainStages chunks in flight; every wait is bounded.
-__global__ void __launch_bounds__(kChainMaxThreads) k_chain(const FrameDev *__restrict__ frames,
+__global__ void __launch_bounds__(kCrowdMaxThreads, 1) k_chain_crowd(const FrameDev *__restrict__ frames,
                                                          const Work *__restrict__ work) {
     const Work wk = work[blockIdx.x];
     const FrameDev &f = frames[wk.frame];
     const int dir = wk.tile & 1;  // 0 = forward (alpha), 1 = backward (beta); bit 1: replay
     const int M = f.M, Mp = f.Mp, MNS = f.MNS, MN = f.MN, n = f.n, N = f.N, xmax = f.xmax;
     const long long rho = f.rho;
-    const int CD = f.chainCD;
+    const int CD = f.crowdCD;
     const int nck = (M + CD - 1) / CD;
-    const int NST = f.chainStages;
+    const int NST = f.crowdStages;
     const int i0 = f.seg_i0, i1 = f.seg_i1;  // symbols of this launch (segment)
     const int send = (int)(rho - (long long)n * N) + xmax;  // state of the end drift
     const bool segm = (f.chain_flags & CH_SEGMENTED) != 0;
@@ -221,9 +188,9 @@ __global__ void __launch_bounds__(kChainMaxThreads) k_chain(const FrameDev *__re
     // this launch's symbols of W (plus the 16-float tail slack), destination
     // inside its stage, 16-byte alignment and size.  A violation records
     // ST_ARG and the chain does not start.
-    __shared__ ChunkTab tab;
+    __shared__ CrowdTab tab;
     for (int k = threadIdx.x; k < nck && k < kMaxChunks; k += blockDim.x) {
-        chunk_geom(f, dir, k, tab);
+        crowd_geom(f, dir, k, tab);
         const bool ok = tab.off[k] + (long long)tab.bytes[k] / 4 <= f.wblk + 16 &&
                         tab.bytes[k] % 16 == 0 && tab.bytes[k] / 4 <= stageFloats;
         if (!ok) atomicExch(&s_fail, ST_ARG);
@@ -266,13 +233,14 @@ __global__ void __launch_bounds__(kChainMaxThreads) k_chain(const FrameDev *__re
     int steps = 0;         // every thread: steps taken in this direction so far
     if (!fresh && segm) {
         const ChainState &cs = f.cst[dir];
-        steps = (int)cs.steps;
+        steps = cs.steps;
         if (threadIdx.x == 0) {
-            theta = (float)cs.theta;
-            mean = (float)cs.mean;
-            ztilt = cs.logZ / 0.6931471805599453;
-            lc_prev = (float)cs.lc_sum;
-            lrow = (float)cs.lrow;
+            theta = cs.theta;
+            mean = cs.mean;
+            zexp = cs.zexp;
+            ztilt = cs.ztilt;
+            lc_prev = cs.lc_sum;
+            lrow = cs.lrow;
             lc_cnt = cs.lc_cnt;
         }
     }
@@ -487,7 +455,8 @@ __global__ void __launch_bounds__(kChainMaxThreads) k_chain(const FrameDev *__re
             ChainState &cs = f.cst[dir];
             cs.theta = theta;
             cs.mean = mean;
-            cs.logZ = ((double)zexp + ztilt) * 0.6931471805599453;
+            cs.zexp = zexp;
+            cs.ztilt = ztilt;
             cs.lc_sum = lc_prev;
             cs.lrow = lrow;
             cs.lc_cnt = lc_cnt;
@@ -789,37 +758,48 @@ cudaError_t launch_pack(const FrameDev *frames, const uint8_t *const *rx_bytes,
 }
 
 size_t chain_smem_bytes(const FrameDev &f) {
-    const size_t stageFloats = ((size_t)(f.chainCD + f.MN + 1) * f.MNS + 8 + 3) & ~(size_t)3;
-    return 4 * (2 * (size_t)f.Mp + (size_t)f.chainStages * stageFloats);
+    const size_t nck = (f.chainVC + f.chainCK - 1) / f.chainCK;
+    // rows, lane groups and their lanes' places, chunk table (8 bytes each, to 16), stages
+    return (size_t)f.chainRing * (f.Mp + 2 * kChainRowPad) * 4 + (size_t)f.chainWarps * f.chainList * sizeof(LaneGroup) +
+           (size_t)f.chainWarps * (f.chainList - 1) * 32 * sizeof(int4) +
+           ((nck * sizeof(ChunkGeom) + 15) & ~(size_t)15) +
+           (size_t)f.chainStages * f.chainStageFloats * 4;
 }
 
-cudaError_t launch_chain(const FrameDev *frames, const Work *work, int nwork, size_t smem,
-                         int threads, cudaStream_t st) {
+// MN with a compiled kernel (launches whose frames share it): n = 4 .. 12, I = 1, 2, 3.
+size_t crowd_smem_bytes(const FrameDev &f) {
+    const size_t stageFloats = ((size_t)(f.crowdCD + f.MN + 1) * f.MNS + 8 + 3) & ~(size_t)3;
+    return 4 * (2 * (size_t)f.Mp + (size_t)f.crowdStages * stageFloats);
+}
+
+cudaError_t launch_chain_crowd(const FrameDev *frames, const Work *work, int nwork, size_t smem,
+                               int threads, cudaStream_t st) {
     if (nwork <= 0) return cudaSuccess;
-    // Raise the opt-in limit to the device maximum, once per device (the
-    // attribute is per device): graphs hold chain launches of several waves
-    // with different sizes, and every one must stay valid.
-    static std::atomic<int> max_dyn[64];  // 0 = not yet set on that device
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    static std::atomic<uint64_t> attr{0};
+    cudaError_t e = smem_optin_once(k_chain_crowd, attr);
     if (e != cudaSuccess) return e;
-    int lim = (dev >= 0 && dev < 64) ? max_dyn[dev].load(std::memory_order_acquire) : 0;
-    if (lim <= 0) {
-        cudaFuncAttributes fa;
-        e = cudaFuncGetAttributes(&fa, k_chain);
-        if (e != cudaSuccess) return e;
-        int optin = 0;
-        e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        if (e != cudaSuccess) return e;
-        lim = optin - (int)fa.sharedSizeBytes;
-        e = cudaFuncSetAttribute(k_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        if (e != cudaSuccess) return e;
-        if (dev >= 0 && dev < 64) max_dyn[dev].store(lim, std::memory_order_release);
-    }
-    if ((long long)smem > lim) return cudaErrorInvalidValue;
-    if (threads != 128 && threads != 256 && threads != 512) threads = kChainThreads;
-    k_chain<<<nwork, threads, smem, st>>>(frames, work);
+    if (threads != 128 && threads != 256 && threads != 512) threads = kCrowdThreads;
+    k_chain_crowd<<<nwork, threads, smem, st>>>(frames, work);
     return cudaGetLastError();
+}
+
+cudaError_t launch_chain(int mn, const FrameDev *frames, const Work *work, int nwork, size_t smem,
+                         int cluster, int threads, cudaStream_t st) {
+    if (nwork <= 0) return cudaSuccess;
+    if (threads < 96 || threads > kChainMaxThreads || threads % 32) return cudaErrorInvalidValue;
+    switch (mn) {
+        case 9: case 11: case 13: case 15: case 16: case 17:
+            return launch_chain_a(mn, frames, work, nwork, smem, cluster, threads, st);
+        case 19: case 21: case 22: case 23: case 25:
+            return launch_chain_b(mn, frames, work, nwork, smem, cluster, threads, st);
+        case 28: case 29: case 31: case 33:
+            return launch_chain_c(mn, frames, work, nwork, smem, cluster, threads, st);
+        case 34: case 37: case 41:
+            return launch_chain_d(mn, frames, work, nwork, smem, cluster, threads, st);
+        case 45: case 49:
+            return launch_chain_e(mn, frames, work, nwork, smem, cluster, threads, st);
+        default: return launch_chain_mn<0>(frames, work, nwork, smem, cluster, threads, st);
+    }
 }
 
 int finalize_chunks(int N) { return (N + kFinChunk - 1) / kFinChunk; }

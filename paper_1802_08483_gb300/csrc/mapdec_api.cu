@@ -187,8 +187,16 @@ constexpr int kPhases = 5;  // pack, forward producers, chains, backward produce
 constexpr int kRegions = 3; // rotating scratch regions when frames need several waves
 constexpr size_t kFwdSmemBudget = 110 * 1024;
 constexpr size_t kBwdSmemBudget = 110 * 1024;  // two CTAs per SM
-constexpr size_t kChainSmemBudget = 100 * 1024;  // two chains per SM
-constexpr int kChainStages = 2;
+constexpr size_t kChainSmemBudget = 100 * 1024;  // two recursion CTAs per SM
+constexpr size_t kChainSmemAlone = 200 * 1024;   // one (k_chain)
+constexpr size_t kChainSmemMost = 220 * 1024;    // beyond what an SM holds: k_chain_crowd
+constexpr int kChainMinGroups = 12;
+
+// What a frame's class asks of the recursions (0 = the planner's choice).
+struct ChainAsk {
+    size_t budget = 0;  // shared memory of one CTA
+    int stages = 0;
+};
 
 struct FrameHost {
     mapdec_frame_desc_t d;
@@ -201,6 +209,7 @@ struct FrameHost {
     size_t scratch_floats = 0;
     double cost = 0.0;
     int segK = 0, nseg = 1; // segmented mode: symbols per segment, segments
+    ChainAsk chain;         // tuned recursion parameters of the frame's class
     bool store = false;     // keep the receiver metrics in HBM for the APP producer
     bool tc = false;        // forward producer on the tensor cores
     bool tcb = false;       // APP producer on the tensor cores
@@ -232,6 +241,45 @@ bool tune_lookup(int q, int n, int I, mapdec_tune_t &out) {
             return true;
         }
     return false;
+}
+
+ChainAsk chain_ask(const mapdec_tune_t *tune) {
+    ChainAsk a;
+    if (tune && tune->chain_budget_kb >= 16 && tune->chain_budget_kb <= 220)
+        a.budget = (size_t)tune->chain_budget_kb * 1024;
+    if (const char *e = std::getenv("MAPDEC_CHAIN_BUDGET_KB")) {  // tuning override
+        const int kb = std::atoi(e);
+        if (kb >= 16 && kb <= 220) a.budget = (size_t)kb * 1024;
+    }
+    if (tune && tune->chain_stages >= 2 && tune->chain_stages <= 8) a.stages = tune->chain_stages;
+    if (const char *e = std::getenv("MAPDEC_CHAIN_STAGES")) {  // tuning override
+        const int v = std::atoi(e);
+        if (v >= 2 && v <= 8) a.stages = v;
+    }
+    return a;
+}
+
+// The order in which k_chain adds a row's states up, a function of the frame's
+// shape alone: equal chunks of states (the fewest whose staged rows of W would
+// fit 100 KB twice, at most 64), each over 256 virtual lanes.  Log-likelihoods
+// and gradients then do not depend on how a launch splits the work.
+void plan_chain_order(FrameDev &f) {
+    auto fits = [&](int cd) {
+        const size_t stage = rup((size_t)(cd + f.MN + 1) * f.MNS + 8, 4);
+        return 4 * (2 * (size_t)f.Mp + 2 * stage) <= 100 * 1024;
+    };
+    int CD = f.M;
+    for (int nck = 1; nck <= 64; ++nck) {
+        CD = (f.M + nck - 1) / nck;
+        if (fits(CD)) break;
+    }
+    f.chainCD = CD;
+    auto groups = [](int nst) { return ((nst << chain_lanes_lg(nst)) + 31) / 32; };
+    const int nck = (f.M + CD - 1) / CD;
+    f.chainVW = groups(CD);
+    const int last = groups(f.M - (nck - 1) * CD);
+    f.chainNV = (nck - 1) * f.chainVW + last;
+    f.chainVWarps = std::min(8, nck > 1 ? std::max(f.chainVW, last) : last);
 }
 
 // Fill shape-dependent fields of dev (P, S, T, nsub, ...) for received length rho.
@@ -328,46 +376,110 @@ void plan_shape(FrameDev &f, const mapdec_frame_desc_t &d, bool grad, int forceP
     f.Pf = f.P;
     f.Sf = f.S;
     f.Tf = f.T;
-    // chain chunk: all states at once if it fits, else the largest power of two;
-    // as many stages in flight as the budget allows (at least two)
-    size_t cbud = kChainSmemBudget;
-    if (tune && tune->chain_budget_kb >= 16 && tune->chain_budget_kb <= 220)
-        cbud = (size_t)tune->chain_budget_kb * 1024;
-    if (const char *e = std::getenv("MAPDEC_CHAIN_BUDGET_KB")) {  // tuning override
-        const int kb = std::atoi(e);
-        if (kb >= 16 && kb <= 220) cbud = (size_t)kb * 1024;
-    }
-    int stages = kChainStages;
-    if (tune && tune->chain_stages >= 2 && tune->chain_stages <= 8) stages = tune->chain_stages;
-    if (const char *e = std::getenv("MAPDEC_CHAIN_STAGES")) {  // tuning override
+    plan_chain_order(f);
+}
+
+// Launches with more recursions than SMs run k_chain_crowd (chain.cu says why).
+bool crowd_launch(long long nwork) {
+    bool crowd = nwork > (device_sms() > 0 ? device_sms() : 152);
+    if (const char *e = std::getenv("MAPDEC_CHAIN_CLUSTER")) crowd = std::atoi(e) == 0;  // testing override
+    return crowd;
+}
+
+// CTAs per recursion for a launch of nwork recursions whose widest row has
+// maxNV lane groups: more while the GPU has idle SMs for them and a CTA keeps
+// at least kChainMinGroups groups (below that the cluster barrier costs more
+// than the split gains).
+int chain_cluster(long long nwork, int maxNV) {
+    int cl = 1;
+    const int sms = device_sms() > 0 ? device_sms() : 152;
+    while (cl < 8 && nwork * cl * 2 <= sms && (maxNV + 2 * cl - 1) / (2 * cl) >= kChainMinGroups)
+        cl *= 2;
+    if (const char *e = std::getenv("MAPDEC_CHAIN_CLUSTER")) {  // testing override
         const int v = std::atoi(e);
-        if (v >= 2 && v <= 8) stages = v;
+        if (v == 1 || v == 2 || v == 4 || v == 8) cl = v;
     }
-    auto chain_fits = [&](int cd, int stg) {
-        FrameDev t = f;
-        t.chainCD = cd;
-        t.chainStages = stg;
-        return chain_smem_bytes(t) <= cbud;
-    };
-    // the fewest chunks per step that fit, equal in size (at most 64 chunks)
-    int CD = f.M;
+    return cl;
+}
+
+// k_chain_crowd's chunks: the fewest per step that fit the budget (100 KB unless
+// tuned) with the stages in flight (two unless tuned), equal in size, at most 64.
+// Untuned they are the summation order's chunks.
+void plan_crowd(FrameDev &f, const ChainAsk &ask) {
+    f.crowdStages = ask.stages ? ask.stages : 2;
+    const size_t bud = ask.budget ? ask.budget : kChainSmemBudget;
     for (int nck = 1; nck <= 64; ++nck) {
-        CD = (f.M + nck - 1) / nck;
-        if (chain_fits(CD, stages)) break;
+        f.crowdCD = (f.M + nck - 1) / nck;
+        if (crowd_smem_bytes(f) <= bud) break;
     }
     if (const char *e = std::getenv("MAPDEC_CHAIN_CD")) {  // tuning / testing override
-        const int cd = std::atoi(e);
+        const int cd = std::atoi(e), own = f.crowdCD;
         if (cd >= 32) {
-            FrameDev t = f;
-            t.chainCD = std::min(cd, f.M);
-            t.chainStages = stages;
-            if (chain_smem_bytes(t) <= 227 * 1024) CD = t.chainCD;
+            f.crowdCD = std::min(cd, f.M);
+            if (crowd_smem_bytes(f) > 227 * 1024) f.crowdCD = own;
         }
     }
-    // at most 64 chunks per step (the chain's chunk table)
-    CD = std::max(CD, (f.M + 63) / 64);
-    f.chainCD = CD;
-    f.chainStages = stages;
+    f.crowdCD = std::max(f.crowdCD, (f.M + 63) / 64);
+}
+
+// A frame's share of a k_chain launch with cl CTAs per recursion: lane
+// groups per CTA, the fewest staged chunks of them that fit the budget with two
+// copies in flight, row buffers, and as many copies in flight as fit (a step is
+// shorter than a copy's latency).
+void plan_chain(FrameDev &f, int cl, int threads, const ChainAsk &ask) {
+    size_t bud = ask.budget;
+    if (bud == 0) bud = kChainSmemAlone;
+    plan_crowd(f, ask);
+    f.chainVC = (f.chainNV + cl - 1) / cl;
+    f.chainWarps = threads / 32 - 2;
+    if (cl == 1 && threads <= 320) {  // narrow: a warp per virtual warp
+        const int nck = (f.M + f.chainCD - 1) / f.chainCD;
+        f.chainList = nck * ((std::max(f.chainVW, f.chainNV - (nck - 1) * f.chainVW) + 7) / 8) + 1;
+    } else {
+        f.chainList = (f.chainVC + f.chainWarps - 1) / f.chainWarps + 1;
+    }
+    const int span = 32 >> chain_lanes_lg(std::min(f.chainCD, f.M));  // states per group, at most
+    auto fits = [&](int ck, int stg, size_t budget) {
+        f.chainCK = ck;
+        f.chainStages = stg;
+        const size_t rowsW = std::min<size_t>((size_t)ck * span + f.MN - 1, f.M);
+        f.chainStageFloats = (int)rup(rowsW * f.MNS + 8, 4);
+        return chain_smem_bytes(f) <= budget;
+    };
+    const int need = ask.stages ? ask.stages : 2;
+    // four rows are summed together, then stored one a step while the next ones
+    // (and a scaled copy of the last) are written.  A row too long for that is
+    // summed, scaled in place and stored at every step.
+    f.chainRing = 9;
+    if ((size_t)f.chainRing * (f.Mp + 2 * kChainRowPad) * 4 > bud / 2) f.chainRing = 2;
+    // rows are not scaled between sums: a step grows them by at most about
+    // 2^{theta n}, theta <= 1.6, which four (two) of them keep within FP32
+    f.chainCap = f.chainRing < 4 ? 1 : (f.n <= 15 ? 4 : 2);
+    int ck = f.chainVC;
+    for (int nck = 1; nck <= f.chainVC; ++nck) {
+        ck = (f.chainVC + nck - 1) / nck;
+        if (fits(ck, need, bud)) break;
+    }
+    if (const char *e = std::getenv("MAPDEC_CHAIN_CD")) {  // tuning / testing override: states
+        const int cd = std::atoi(e);
+        if (cd >= 32) {
+            const int k = std::max(1, std::min(cd / span, f.chainVC));
+            if (fits(k, need, 220 * 1024)) ck = k;
+        }
+    }
+    int stages = need;
+    if (!ask.stages)
+        while (stages < 8 && fits(ck, stages + 1, bud)) ++stages;
+    fits(ck, stages, bud);
+}
+
+// Block size of a recursion launch over frames with at most maxVW virtual warps
+// and maxNV lane groups: a warp per virtual warp while no warp then has more than
+// one group, else (and in clusters) a warp per lane group up to 14; and the two
+// that move data.
+int chain_threads(int cl, int maxVW, int maxNV) {
+    if (cl == 1 && maxNV <= 8) return 32 * (maxVW + 2);
+    return 32 * (std::max(9, std::min(14, (maxNV + cl - 1) / cl)) + 2);
 }
 
 // Forward tile of the tensor-core producer: up to two lattices per thread
@@ -529,12 +641,23 @@ struct SegLaunch {
     cudaEvent_t ev_fwd2 = nullptr, ev_chain2 = nullptr, ev_bwd = nullptr;  // recompute sweep
 };
 
+// Recursions of a wave's frames with one MN.
+struct ChainLaunch {
+    int mn = 0;
+    Work *d_work = nullptr; int n = 0; size_t smem = 0;
+};
+constexpr int kMaxChainStreams = 6;  // launches per MN side by side, else one for all frames
+
 struct Wave {
     int f0 = 0, f1 = 0;
     std::vector<SegLaunch> segs;  // segmented mode
     FrameDev *d_frames = nullptr;
     std::vector<ClassLaunch> cls;
-    Work *d_chain = nullptr; int nchain = 0; size_t smem_chain = 0;
+    std::vector<ChainLaunch> chains;  // the recursions, a launch per MN (or one for all)
+    size_t smem_chain = 0;            // of the widest frame
+    bool crowd = false;               // more recursions than SMs (k_chain_crowd)
+    int chain_cl = 1, chain_thr = 0;  // CTAs per recursion, block size
+    int chain_mn = 0;                 // MN of every frame, 0 where they differ
     Work *d_fin = nullptr; int nfin = 0;
     const uint8_t **d_rxptr = nullptr;
     uint32_t **d_rxwptr = nullptr;
@@ -570,6 +693,8 @@ struct mapdec_batch {
     size_t region_floats = 0;    // stride between rotating scratch regions
     int regions = 1;
     cudaStream_t aux_stream = nullptr;  // chains run here, overlapping the producers
+    std::vector<cudaStream_t> chain_streams;  // and here, a wave's further chain launches
+    std::vector<cudaEvent_t> chain_done;
     std::vector<cudaEvent_t> dep;       // per wave: forward done, chains done
     std::vector<Wave> waves;
     std::vector<void *> allocs;
@@ -598,6 +723,8 @@ struct mapdec_batch {
         for (cudaEvent_t e : seg_events) cudaEventDestroy(e);
         if (cap_stream) cudaStreamDestroy(cap_stream);
         if (aux_stream) cudaStreamDestroy(aux_stream);
+        for (cudaStream_t t : chain_streams) cudaStreamDestroy(t);
+        for (cudaEvent_t e : chain_done) cudaEventDestroy(e);
         for (cudaEvent_t e : dep) cudaEventDestroy(e);
 
         for (void *p : allocs) cudaFree(p);
@@ -787,6 +914,7 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
         mapdec_tune_t tu{};
         const bool tuned = !plain && tune_lookup(h.d.q, h.d.n, h.d.I, tu);
         plan_shape(h.dev, h.d, b->grad, plain ? 0 : forceP, tuned ? &tu : nullptr);
+        h.chain = chain_ask(tuned ? &tu : nullptr);
         h.store = tuned && tu.store_metric == 1;
         if (const char *e = std::getenv("MAPDEC_STORE_R")) h.store = std::atoi(e) == 1;  // testing
         if (plain || b->grad || (flags & MAPDEC_BATCH_SEGMENTED)) h.store = false;
@@ -935,7 +1063,6 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
     b->d_scratch = (float *)b->dalloc(b->region_floats * 4 * b->regions + 256);
     // per-wave descriptors and work tables
     const bool segmented = b->segmented;
-    if (const char *e = std::getenv("MAPDEC_CHAIN_THREADS")) b->chain_threads = std::atoi(e);  // A/B override
     for (size_t wi = 0; wi < b->waves.size(); ++wi) {
         Wave &w = b->waves[wi];
         size_t off = (wi % b->regions) * b->region_floats;
@@ -943,8 +1070,23 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
         std::vector<const uint8_t *> rxp;
         std::vector<uint32_t *> rxwp;
         std::map<ClassKey, std::vector<int>> byclass;
+        // both directions of every frame in one launch
+        const long long nrec = 2LL * (w.f1 - w.f0);
+        int maxNV = 0, maxVW = 0;
+        for (int i = w.f0; i < w.f1; ++i) {
+            maxNV = std::max(maxNV, b->fr[i].dev.chainNV);
+            maxVW = std::max(maxVW, b->fr[i].dev.chainVWarps);
+        }
+        w.chain_mn = b->fr[w.f0].dev.MN;
+        for (int i = w.f0; i < w.f1; ++i)
+            if (b->fr[i].dev.MN != w.chain_mn) w.chain_mn = 0;
+        w.chain_cl = chain_cluster(nrec, maxNV);
+        w.crowd = crowd_launch(b->waves.size() > 1 ? 1 << 20 : nrec);
+        w.chain_thr = chain_threads(w.chain_cl, maxVW, maxNV);
         for (int i = w.f0; i < w.f1; ++i) {
             FrameHost &h = b->fr[i];
+            plan_chain(h.dev, w.chain_cl, w.chain_thr, h.chain);
+            if (chain_smem_bytes(h.dev) > kChainSmemMost) w.crowd = true;  // rows too long for k_chain
             FrameDev f = h.dev;
             f.rxbits = b->d_rxw + h.rxw_off;
             f.cw = b->d_cw + h.cw_off;
@@ -1030,12 +1172,31 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
             return (double)devs[a].N * devs[a].M * devs[a].MN >
                    (double)devs[c].N * devs[c].M * devs[c].MN;
         });
-        std::vector<Work> chain;
-        size_t csm = 0;
-        for (int k : order) {
-            chain.push_back({k, 0});
-            chain.push_back({k, 1});
-            csm = std::max(csm, chain_smem_bytes(devs[k]));
+        {
+            // a launch per MN runs that MN's compiled kernel; segmented waves keep
+            // one launch per segment
+            std::map<int, std::vector<Work>> per;
+            std::map<int, size_t> csm;
+            for (int k : order) per[devs[k].MN];
+            const bool apart = !segmented && !w.crowd && (int)per.size() <= kMaxChainStreams;
+            per.clear();
+            for (int k : order) {
+                const int mn = apart ? devs[k].MN : w.chain_mn;
+                per[mn].push_back({k, 0});
+                per[mn].push_back({k, 1});
+                csm[mn] = std::max(csm[mn], w.crowd ? crowd_smem_bytes(devs[k]) : chain_smem_bytes(devs[k]));
+                w.smem_chain = std::max(w.smem_chain, csm[mn]);
+            }
+            for (auto &kv : per) {
+                ChainLaunch c;
+                c.mn = kv.first;
+                c.n = (int)kv.second.size();
+                c.smem = csm[kv.first];
+                c.d_work = (Work *)b->dalloc(sizeof(Work) * kv.second.size());
+                CK(cudaMemcpy(c.d_work, kv.second.data(), sizeof(Work) * kv.second.size(),
+                              cudaMemcpyHostToDevice));
+                w.chains.push_back(c);
+            }
         }
         {
             std::vector<Work> fin;
@@ -1045,10 +1206,6 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
             w.d_fin = (Work *)b->dalloc(sizeof(Work) * fin.size());
             CK(cudaMemcpy(w.d_fin, fin.data(), sizeof(Work) * fin.size(), cudaMemcpyHostToDevice));
         }
-        w.nchain = (int)chain.size();
-        w.smem_chain = csm;
-        w.d_chain = (Work *)b->dalloc(sizeof(Work) * chain.size());
-        CK(cudaMemcpy(w.d_chain, chain.data(), sizeof(Work) * chain.size(), cudaMemcpyHostToDevice));
         for (auto &kv : byclass) {
             ClassLaunch c;
             c.n = std::get<0>(kv.first);
@@ -1077,6 +1234,16 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
         if (segmented) build_segments(b, w, devs, byclass);
     }
     CK(cudaStreamCreateWithFlags(&b->aux_stream, cudaStreamNonBlocking));
+    size_t nch = 1;
+    for (const Wave &w : b->waves) nch = std::max(nch, w.chains.size());
+    for (size_t k = 1; k < nch; ++k) {
+        cudaStream_t t = nullptr;
+        CK(cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking));
+        b->chain_streams.push_back(t);
+        cudaEvent_t e = nullptr;
+        CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+        b->chain_done.push_back(e);
+    }
     b->dep.resize(b->waves.size() * 2 + 2);
     for (auto &e : b->dep) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     if (flags & MAPDEC_BATCH_TIMING) {
@@ -1085,6 +1252,12 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
         for (auto &e : b->events) CK(cudaEventCreate(&e));
     }
     return MAPDEC_OK;
+}
+
+cudaError_t run_chain(const mapdec_batch *b, const Wave &w, int mn, const FrameDev *frames, const Work *work,
+                      int n, size_t smem, cudaStream_t st) {
+    return w.crowd ? launch_chain_crowd(frames, work, n, smem, b->chain_threads, st)
+                   : launch_chain(mn, frames, work, n, smem, w.chain_cl, w.chain_thr, st);
 }
 
 // Enqueue one full run on stream st (producers) and the batch's auxiliary
@@ -1138,8 +1311,18 @@ int64_t enqueue_run(mapdec_batch *b, bool grad, cudaStream_t st) {
         // chains of wave w on the auxiliary stream
         CK(cudaStreamWaitEvent(cs, b->dep[2 * w], 0));
         mark(w, 2, 0, cs);
-        CK(launch_chain(wv.d_frames, wv.d_chain, wv.nchain, wv.smem_chain, b->chain_threads, cs));
-        ++launches;
+        // further launches (other MN) side by side on streams of their own
+        for (size_t k = 1; k < wv.chains.size(); ++k) {
+            cudaStream_t ck = b->chain_streams[k - 1];
+            CK(cudaStreamWaitEvent(ck, b->dep[2 * w], 0));
+            const ChainLaunch &c = wv.chains[k];
+            CK(run_chain(b, wv, c.mn, wv.d_frames, c.d_work, c.n, c.smem, ck));
+            CK(cudaEventRecord(b->chain_done[k - 1], ck));
+        }
+        CK(run_chain(b, wv, wv.chains[0].mn, wv.d_frames, wv.chains[0].d_work, wv.chains[0].n,
+                     wv.chains[0].smem, cs));
+        for (size_t k = 1; k < wv.chains.size(); ++k) CK(cudaStreamWaitEvent(cs, b->chain_done[k - 1], 0));
+        launches += (int64_t)wv.chains.size();
         mark(w, 2, 1, cs);
         CK(cudaEventRecord(b->dep[2 * w + 1], cs));
     };
@@ -1225,7 +1408,7 @@ int64_t enqueue_run_seg(mapdec_batch *b, bool grad, cudaStream_t st) {
             fwd(sl);
             CK(cudaEventRecord(sl.ev_fwd, st));
             CK(cudaStreamWaitEvent(cs, sl.ev_fwd, 0));
-            CK(launch_chain(sl.d_frames, sl.d_rec, sl.nrec, wv.smem_chain, b->chain_threads, cs));
+            CK(run_chain(b, wv, wv.chain_mn, sl.d_frames, sl.d_rec, sl.nrec, wv.smem_chain, cs));
             ++launches;
             CK(cudaEventRecord(sl.ev_rec, cs));
         }
@@ -1242,7 +1425,7 @@ int64_t enqueue_run_seg(mapdec_batch *b, bool grad, cudaStream_t st) {
             CK(cudaStreamWaitEvent(cs, sl.ev_fwd2, 0));
             // alpha/beta buffer s % 2 was last read by the APP producers of segment s+2
             if (s + 2 < S) CK(cudaStreamWaitEvent(cs, wv.segs[s + 2].ev_bwd, 0));
-            CK(launch_chain(sl.d_frames, sl.d_bw, sl.nbw, wv.smem_chain, b->chain_threads, cs));
+            CK(run_chain(b, wv, wv.chain_mn, sl.d_frames, sl.d_bw, sl.nbw, wv.smem_chain, cs));
             ++launches;
             CK(cudaEventRecord(sl.ev_chain2, cs));
         };
@@ -1907,6 +2090,10 @@ int mapdec_decode_noalloc(const mapdec_frame_desc_t *frame, const uint8_t *rx_de
     FrameDev f{};
     plan_shape(f, d, false, 0);
     split_supertiles(f, supertile_split(most_supertiles(f)));
+    const int cl = chain_cluster(2, f.chainNV);
+    const int cthr = chain_threads(cl, f.chainVWarps, f.chainNV);
+    plan_chain(f, cl, cthr, chain_ask(nullptr));
+    const bool crowd = crowd_launch(2) || chain_smem_bytes(f) > kChainSmemMost;
     // carve the arena (every region 256-byte aligned)
     size_t off = 0;
     auto take = [&](size_t bytes) -> size_t {
@@ -1971,7 +2158,9 @@ int mapdec_decode_noalloc(const mapdec_frame_desc_t *frame, const uint8_t *rx_de
         e = launch_pack(fdev, (const uint8_t *const *)(A + o_rxp), (uint32_t *const *)(A + o_rxwp), 1,
                         nwords, s);
     if (e == cudaSuccess) e = launch_fwd(d.n, d.I, fdev, wf, f.Tf, fwd_smem_bytes(f), s);
-    if (e == cudaSuccess) e = launch_chain(fdev, wc, 2, chain_smem_bytes(f), 0, s);
+    if (e == cudaSuccess)
+        e = crowd ? launch_chain_crowd(fdev, wc, 2, crowd_smem_bytes(f), 0, s)
+                  : launch_chain(f.MN, fdev, wc, 2, chain_smem_bytes(f), cl, cthr, s);
     if (e == cudaSuccess) e = launch_bwd(d.n, d.I, false, fdev, wb, f.T2, bwd_smem_bytes(f, false), s);
     if (e == cudaSuccess) e = launch_finalize(fdev, wfin, nfin, 1, 0, s);
     int status = MAPDEC_OK;

@@ -33,10 +33,11 @@ enum : int {
 
 // Chain state carried between the segment launches of a frame (segmented mode).
 struct ChainState {
-    double theta, mean, logZ, lc_sum, lrow;
-    int lc_cnt;
-    int pad;
-    long long steps;
+    long long zexp;  // log2 Z of the boundary row: integer part and tilt terms
+    double ztilt;
+    float theta, mean;         // tilt and mean drift of the boundary row
+    float lc_sum, lrow;        // log2 growth since the last tilt update, log2 of the row sum
+    int lc_cnt, steps;         // steps in lc_sum, and in all
 };
 
 // One frame as the kernels see it.  All pointers are device pointers.
@@ -68,8 +69,16 @@ struct FrameDev {
     int nsub;     // sub-tiles per backward super-tile
     int S2;       // max symbols touched by one super-tile (rows of Lp per super-tile)
     int T2;       // backward super-tiles: ceil(T / nsub)
-    int chainCD;  // destination/source states per chain chunk
-    int chainStages;  // chunks in flight (ring of bulk-copy stages), <= 8
+    // Recursions (k_chain).  Summation order: chunks of chainCD states, chainVW
+    // groups of 32 lanes each (the last may differ), chainNV groups in all.
+    int chainCD, chainVW, chainNV;
+    int crowdCD, crowdStages;  // k_chain_crowd: states per staged chunk, chunks in flight
+    // Work split: groups per CTA of the cluster and per staged chunk, copy
+    // stages (<= 8) of chainStageFloats floats, row buffers
+    int chainVC, chainCK, chainStages, chainStageFloats, chainRing;
+    int chainCap;     // rows summed together, at most
+    int chainVWarps;  // virtual warps with lanes (<= 8)
+    int chainWarps, chainList;  // compute warps of the launch, lane groups of one (and an end mark)
     uint32_t wait_limit;  // polls before a recursion's wait on a copy gives up (ST_TIMEOUT)
     int test_flags;       // TEST_SKIP_FIRST_COPY: the first copy is never issued (tests the timeout path)
     long long rho;
@@ -122,6 +131,16 @@ struct FrameDev {
     double *dchan;   // 3 or null
     int *status;     // 1
 };
+
+constexpr int kChainRowPad = 96;  // zeros on both sides of a row (k_chain reads the band past it)
+
+// Lanes that share a state in a chunk of nst states (k_chain's summation order
+// over 256 virtual lanes): 2^lg of them.
+__host__ __device__ inline int chain_lanes_lg(int nst) {
+    int lg = 0;
+    while (lg < 3 && (nst << (lg + 1)) <= 256) ++lg;
+    return lg;
+}
 
 // Work item of a producer launch: (frame, tile).
 struct Work { int frame; int tile; };

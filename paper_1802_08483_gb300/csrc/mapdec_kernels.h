@@ -82,9 +82,25 @@ cudaError_t launch_pack(const FrameDev *frames, const uint8_t *const *rx_bytes,
                         uint32_t *const *rx_words, int nframes, long long max_words,
                         cudaStream_t st);
 size_t chain_smem_bytes(const FrameDev &f);
-// threads: 128, 256 or 512 (anything else selects the default, 256)
-cudaError_t launch_chain(const FrameDev *frames, const Work *work, int nwork, size_t smem,
-                         int threads, cudaStream_t st);
+// cluster: CTAs per recursion (1, 2, 4 or 8); threads: a multiple of 32 from 96 to
+// 512 (the last two warps move data, the others compute; one CTA of more than
+// 320: a warp per lane group instead of one per virtual warp)
+// Recursions of launches with more of them than SMs; threads 128, 256 or 512
+// (anything else: 256).
+size_t crowd_smem_bytes(const FrameDev &f);
+cudaError_t launch_chain_crowd(const FrameDev *frames, const Work *work, int nwork, size_t smem,
+                               int threads, cudaStream_t st);
+// mn: the frames' common MN, 0 where they differ (or always: the general kernel)
+cudaError_t launch_chain(int mn, const FrameDev *frames, const Work *work, int nwork, size_t smem,
+                         int cluster, int threads, cudaStream_t st);
+#define MAPDEC_DECLARE_CHAIN(G)                                                              \
+    cudaError_t launch_chain_##G(int mn, const FrameDev *frames, const Work *work, int nwork, \
+                                 size_t smem, int cluster, int threads, cudaStream_t st);
+MAPDEC_DECLARE_CHAIN(a)
+MAPDEC_DECLARE_CHAIN(b)
+MAPDEC_DECLARE_CHAIN(c)
+MAPDEC_DECLARE_CHAIN(d)
+MAPDEC_DECLARE_CHAIN(e)
 cudaError_t launch_finalize(const FrameDev *frames, const Work *work, int nwork, int nframes,
                             int grad, cudaStream_t st, bool reduce = true);
 size_t chain_state_bytes();
