@@ -542,7 +542,9 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(const FrameDev *__rest
     __shared__ double red[3][kFinThreads / 32];
     if (*f.status != ST_OK) return;
     const int q = f.q, n = f.n, xmax = f.xmax, S2 = f.S2, psT = f.psT;
-    const long long P2 = (long long)f.P * f.nsub;
+    // positions per row tile; row tiles whose sums are added first (gradients)
+    const long long P2 = (long long)f.P * (f.group ? 1 : f.nsub);
+    const int group = max(1, f.group);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const float *Lp = f.Lp;
     const int c0 = f.seg_i0 + (wk.tile - f.fin_base) * kFinChunk;
@@ -575,7 +577,8 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(const FrameDev *__rest
     // unnormalised sums L^u(D) (eq. L without the prior), lane = D mod 32
     auto lsum = [&](int k, int D) {
         const long long lo = __shfl_sync(0xffffffffu, tlo, 4 * k), hi = __shfl_sync(0xffffffffu, thi, 4 * k);
-        float v = 0.f;
+        float v = 0.f, part = 0.f;
+        int left = group - (int)((unsigned)lo % (unsigned)group);  // row tiles left of the group
         for (int t0 = 0; t0 <= hi - lo; t0 += 32) {
             // up to four rows from the start, more found a warp's width at a time
             long long r = myrow;
@@ -584,10 +587,15 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(const FrameDev *__rest
             const int cnt = (int)min(32LL, hi - lo + 1 - t0);
             for (int t = 0; t < cnt; ++t) {
                 const long long row = __shfl_sync(0xffffffffu, r, wide ? t : 4 * k + t);
-                if (D < q) v += Lp[row * q + D];
+                if (D < q) part += Lp[row * q + D];
+                if (--left == 0) {
+                    v += part;
+                    part = 0.f;
+                    left = group;
+                }
             }
         }
-        return v;
+        return v + part;
     };
     // pass 1: z = sum_D prior(D) L^u(D) and, for the extrinsic output, zu = sum_D L^u(D)
     float lu[kFinSym][kFinRegs];
@@ -662,11 +670,20 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(const FrameDev *__rest
             const double Pt = f.dPt, Ps = f.dPs, Pd = f.dPd, k = f.kappa;
             const double Qm = k * Pt * (1.0 - Ps), Qs = k * Pt * Ps;
             double Sw = 0.0, Sd = 0.0, Ss = 0.0;
+            float pw = 0.f, pd = 0.f, ps = 0.f;
+            int left = group - (int)((unsigned)tlo % (unsigned)group);
             for (long long t = tlo; t <= thi; ++t) {
                 const float *gp = f.Gp + row_of(i0 + mine, t) * 3;
-                Sw += gp[0];
-                Sd += gp[1];
-                Ss += gp[2];
+                pw += gp[0];
+                pd += gp[1];
+                ps += gp[2];
+                if (--left == 0 || t == thi) {
+                    Sw += pw;
+                    Sd += pd;
+                    Ss += ps;
+                    pw = pd = ps = 0.f;
+                    left = group;
+                }
             }
             // Sw, Sd, Ss: sums with dR~/dw', dR~/dPd, dR~/dQ's.  R~ is homogeneous
             // of degree n in (Pd, Q'm, Q's) (every bit is deleted or transmitted),

@@ -541,13 +541,17 @@ bool plan_bwd_tc(FrameDev &f) {
     return false;
 }
 
+// Tiles with rows of APP partial sums of their own, and their positions.
+size_t row_tiles(const FrameDev &f) { return f.group ? f.T : f.T2; }
+long long row_positions(const FrameDev &f) { return (long long)f.P * (f.group ? 1 : f.nsub); }
+
 size_t frame_scratch_floats(const FrameDev &f, bool grad) {
     size_t s = 0;
     if (f.Pgroups) s += rup(prior_split_bytes(f) / 4, 64);  // priors split for the tensor cores
     s += rup((size_t)f.N * f.wblk + 16, 64);             // W (+ tail slack for bulk copies)
     s += rup((size_t)(f.N + 1) * f.Mp, 64) * 2;          // alpha, beta
-    s += rup((size_t)f.T2 * f.S2 * f.q, 64);             // Lp
-    if (grad) s += rup((size_t)f.T2 * f.S2 * 3, 64);     // Gp
+    s += rup(row_tiles(f) * f.S2 * f.q, 64);             // Lp
+    if (grad) s += rup(row_tiles(f) * f.S2 * 3, 64);     // Gp
     s += 3 * rup((size_t)(f.N + 1) * 2, 64);             // thf, mcf, thb (doubles)
     if (grad) s += rup((size_t)finalize_chunks(f.N) * 3 * 2, 64);  // Gc (doubles)
     return s;
@@ -555,12 +559,11 @@ size_t frame_scratch_floats(const FrameDev &f, bool grad) {
 
 // Segmented mode: W, alpha, beta and the APP partials for one segment of K
 // symbols, plus forward checkpoints every K symbols.
-int seg_supertiles(const FrameDev &f, int K) {
-    const long long P2 = (long long)f.P * f.nsub;
-    return (int)(((long long)f.n * K + 2LL * f.xmax) / P2 + 3);
+int seg_row_tiles(const FrameDev &f, int K) {
+    return (int)(((long long)f.n * K + 2LL * f.xmax) / row_positions(f) + 3);
 }
 size_t frame_scratch_floats_seg(const FrameDev &f, int K, int S, bool grad) {
-    const int T2s = seg_supertiles(f, K);
+    const int T2s = seg_row_tiles(f, K);
     const int cps = finalize_chunks(K);
     size_t s = 0;
     if (f.Pgroups) s += rup(prior_split_bytes(f) / 4, 64);  // priors split for the tensor cores
@@ -774,9 +777,8 @@ void build_segments(mapdec_batch *b, Wave &w, const std::vector<FrameDev> &devs,
             if (s >= h.nseg) continue;
             FrameDev f = devs[k];
             const int K = h.segK, i0 = s * K, i1 = std::min(f.N, i0 + K);
-            const long long P2 = (long long)f.P * f.nsub;
             const long long plo = std::max(0LL, (long long)f.n * i0 - f.xmax);
-            const long long t2first = plo / P2;
+            const long long t2first = plo / row_positions(f);
             auto shift = [](void *p, long long bytes) {
                 return (void *)((char *)p - bytes);
             };
@@ -977,8 +979,15 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
         }
         h.split = !b->grad && !per_sym && !h.tcb && !(tuned && tu.nsub > 0) &&
                   !std::getenv("MAPDEC_FORCE_NSUB");
+        if (b->grad && !per_sym) {
+            // partial sums per sub-tile; the order of the sums stays that of the
+            // planned super-tiles
+            h.dev.group = h.dev.nsub;
+            h.dev.S2 = h.dev.S;
+            class_ctas[{h.d.n, h.d.I}] += b->segmented ? seg_row_tiles(h.dev, h.segK) - 2 : h.dev.T;
+        }
         if (h.split)
-            class_ctas[{h.d.n, h.d.I}] += b->segmented ? seg_supertiles(h.dev, h.segK) - 2
+            class_ctas[{h.d.n, h.d.I}] += b->segmented ? seg_row_tiles(h.dev, h.segK) - 2
                                                        : most_supertiles(h.dev);
         h.cost = frame_cost(h.dev);
         h.rx_off = b->rx_total;
@@ -994,6 +1003,12 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
     }
     for (auto &h : b->fr) {
         if (h.split) split_supertiles(h.dev, supertile_split(class_ctas[{h.d.n, h.d.I}]));
+        if (h.dev.group) {  // eight CTAs per SM, no more sub-tiles each than planned
+            const int sms = device_sms() > 0 ? device_sms() : 152;
+            h.dev.nsub = (int)std::max(1LL, std::min<long long>(
+                h.dev.group, class_ctas[{h.d.n, h.d.I}] / (8LL * sms)));
+            h.dev.T2 = (h.dev.T + h.dev.nsub - 1) / h.dev.nsub;
+        }
         if (b->segmented) {
             h.scratch_floats = frame_scratch_floats_seg(h.dev, h.segK, h.nseg, b->grad);
         } else {
@@ -1104,9 +1119,9 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
                 f.W = base + o; o += rup((size_t)f.N * f.wblk + 16, 64);
                 f.alpha = base + o; o += rup((size_t)(f.N + 1) * f.Mp, 64);
                 f.beta = base + o; o += rup((size_t)(f.N + 1) * f.Mp, 64);
-                f.Lp = base + o; o += rup((size_t)f.T2 * f.S2 * f.q, 64);
+                f.Lp = base + o; o += rup(row_tiles(f) * f.S2 * f.q, 64);
                 f.Gp = nullptr;
-                if (b->grad) { f.Gp = base + o; o += rup((size_t)f.T2 * f.S2 * 3, 64); }
+                if (b->grad) { f.Gp = base + o; o += rup(row_tiles(f) * f.S2 * 3, 64); }
                 f.thf = (double *)(base + o); o += rup((size_t)(f.N + 1) * 2, 64);
                 f.mcf = (double *)(base + o); o += rup((size_t)(f.N + 1) * 2, 64);
                 f.thb = (double *)(base + o); o += rup((size_t)(f.N + 1) * 2, 64);
@@ -1117,7 +1132,7 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
             } else {
                 // buffers of one segment; per-segment descriptors shift their bases
                 const int K = h.segK, S = h.nseg;
-                const int T2s = seg_supertiles(f, K), cps = finalize_chunks(K);
+                const int T2s = seg_row_tiles(f, K), cps = finalize_chunks(K);
                 // W, alpha and beta twice: segment s uses buffer s % 2, so a
                 // segment's producers overlap the neighbouring segment's recursions
                 f.W = base + o; o += 2 * rup((size_t)K * f.wblk + 16, 64);

@@ -66,9 +66,12 @@ struct FrameDev {
     // index m + xmax) replacing alpha_0 = [m = 0] and beta_N = [m = rho - tau];
     // null for an isolated frame.
     const float *phi0, *phiN;
-    int nsub;     // sub-tiles per backward super-tile
-    int S2;       // max symbols touched by one super-tile (rows of Lp per super-tile)
+    int nsub;     // sub-tiles per backward super-tile (the work of one CTA)
     int T2;       // backward super-tiles: ceil(T / nsub)
+    int group;    // gradient mode: the APP producer keeps the partial sums of every
+                  // sub-tile, and finalize adds them up group sub-tiles at a time;
+                  // 0: the partial sums of a super-tile
+    int S2;       // rows of Lp per sub-tile (group > 0) or super-tile: the symbols it touches
     // Recursions (k_chain).  Summation order: chunks of chainCD states, chainVW
     // groups of 32 lanes each (the last may differ), chainNV groups in all.
     int chainCD, chainVW, chainNV;
@@ -102,8 +105,8 @@ struct FrameDev {
     float *W;        // N * wblk: W_i(s', j) = sum_D prior_i(D) R[p][D][j] at i*wblk + s'*MNS + j
     float *alpha;    // (N+1) * Mp normalised forward rows
     float *beta;     // (N+1) * Mp normalised backward rows
-    float *Lp;       // T2 * S2 * q  partial unnormalised APP sums per super-tile
-    float *Gp;       // T2 * S2 * 3  partial tangent sums per super-tile (gradient mode)
+    float *Lp;       // S2 * q  partial unnormalised APP sums per sub- or super-tile
+    float *Gp;       // S2 * 3  partial tangent sums per sub-tile (gradient mode)
     float *Rout;     // receiver-metric dump (debug entry), (rho+1)*q*MN or null
     float *Rg;       // stored receiver metrics (or null: recompute), T * P*MN * DS:
                      // tile t at t*P*MN*DS, row pl*MN + j, column D (DS = roundup4(q))
