@@ -541,101 +541,113 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(const FrameDev *__rest
     const FrameDev &f = frames[wk.frame];
     __shared__ double red[3][kFinThreads / 32];
     if (*f.status != ST_OK) return;
-    const int q = f.q, n = f.n, xmax = f.xmax, S2 = f.S2, psT = f.psT;
+    const int q = f.q, n = f.n, xmax = f.xmax, S2 = f.S2, psT = f.psT, seg0 = f.seg_i0;
+    const bool ps = f.ps != 0;
     // positions per row tile; row tiles whose sums are added first (gradients)
     const long long P2 = (long long)f.P * (f.group ? 1 : f.nsub);
-    const int group = max(1, f.group);
+    const unsigned group = max(1, f.group);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const float *Lp = f.Lp;
-    const int c0 = f.seg_i0 + (wk.tile - f.fin_base) * kFinChunk;
+    const float *__restrict__ Lp = f.Lp;
+    const float *__restrict__ priors = f.priors;
+    float *const app = f.app, *const dpri = f.dpriors, *const ext = f.ext;
+    const int c0 = seg0 + (wk.tile - f.fin_base) * kFinChunk;
     const int i1 = min(f.seg_i1, c0 + kFinChunk);
     const int i0 = c0 + warp * kFinSym;
     const int ns = max(0, min(kFinSym, i1 - i0));  // symbols of this warp
-    // Rows of the APP partials of symbol i0 + k: tiles tlo .. thi, one row each.
-    // The lanes of symbol k find theirs; row of tile t: t S2 + i - (the tile's
-    // first symbol), or t itself (per-symbol producers: rows are work items).
+    // Rows of the APP partials of symbol i0 + k: tiles tlo .. tlo + cnt - 1, one row
+    // each, looked up by lanes 4 k .. 4 k + 3.  Row of tile t: t S2 + i - (the
+    // tile's first symbol), or t itself (per-symbol producers: rows are work items).
     const int mine = lane >> 2;
-    long long tlo = 0, thi = -1;
+    long long tlo = 0;
+    int cnt = 0;
     if (mine < ns) {
         const int i = i0 + mine;
-        if (f.ps) {
+        if (ps) {
             tlo = (long long)i * psT;
-            thi = tlo + psT - 1;
+            cnt = psT;
         } else {
             tlo = max(0LL, (long long)n * i - xmax) / P2;
-            thi = min(f.rho, (long long)n * i + xmax) / P2;
+            cnt = (int)(min(f.rho, (long long)n * i + xmax) / P2 - tlo) + 1;
         }
     }
+    const int most = __reduce_max_sync(0xffffffffu, cnt);
     auto row_of = [&](int i, long long t) -> long long {
-        if (f.ps) return t;
+        if (ps) return t;
         // i - ceil((t P2 - xmax) / n), the tile's first symbol not before the segment's
         const unsigned past = (unsigned)((long long)n * i - t * P2 + xmax) / (unsigned)n;
-        return t * S2 + min(i - f.seg_i0, (int)past);
+        return t * S2 + min(i - seg0, (int)past);
     };
-    // the first four rows of each symbol, one per lane
-    const long long myrow = mine < ns && tlo + (lane & 3) <= thi ? row_of(i0 + mine, tlo + (lane & 3)) : 0;
-    // unnormalised sums L^u(D) (eq. L without the prior), lane = D mod 32
-    auto lsum = [&](int k, int D) {
-        const long long lo = __shfl_sync(0xffffffffu, tlo, 4 * k), hi = __shfl_sync(0xffffffffu, thi, 4 * k);
-        float v = 0.f, part = 0.f;
-        int left = group - (int)((unsigned)lo % (unsigned)group);  // row tiles left of the group
-        for (int t0 = 0; t0 <= hi - lo; t0 += 32) {
-            // up to four rows from the start, more found a warp's width at a time
-            long long r = myrow;
-            const bool wide = hi - lo > 3;
-            if (wide) r = lo + t0 + lane <= hi ? row_of(i0 + k, lo + t0 + lane) : 0;
-            const int cnt = (int)min(32LL, hi - lo + 1 - t0);
-            for (int t = 0; t < cnt; ++t) {
-                const long long row = __shfl_sync(0xffffffffu, r, wide ? t : 4 * k + t);
-                if (D < q) part += Lp[row * q + D];
-                if (--left == 0) {
-                    v += part;
-                    part = 0.f;
-                    left = group;
+    // Unnormalised sums L^u(D) (eq. L without the prior) of the warp's symbols at
+    // D = D0 + lane, the rows of a symbol in order.  Four rows of every symbol are
+    // loaded at a time: one symbol after another a warp waited for memory 2 to 40
+    // times each (N = 50, q = 16: 22000 clocks of 36000).
+    auto lsums = [&](int D0, float (&v)[kFinSym]) {
+        const int D = D0 + lane;
+        float part[kFinSym];
+#pragma unroll
+        for (int k = 0; k < kFinSym; ++k) v[k] = part[k] = 0.f;
+        for (int t0 = 0; t0 < most; t0 += 4) {
+            const int t = t0 + (lane & 3);
+            const long long row = t < cnt ? row_of(i0 + mine, tlo + t) : -1;
+            // rows that end a group (or the symbol's range)
+            const unsigned last =
+                __ballot_sync(0xffffffffu, (unsigned)(tlo + t) % group == group - 1 || t + 1 == cnt);
+            float x[kFinSym][4];
+#pragma unroll
+            for (int k = 0; k < kFinSym; ++k)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const long long r = __shfl_sync(0xffffffffu, row, 4 * k + e);
+                    x[k][e] = r >= 0 && D < q ? Lp[r * q + D] : 0.f;
                 }
-            }
+#pragma unroll
+            for (int k = 0; k < kFinSym; ++k)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    part[k] += x[k][e];
+                    if (last >> (4 * k + e) & 1u) {
+                        v[k] += part[k];
+                        part[k] = 0.f;
+                    }
+                }
         }
-        return v + part;
     };
     // pass 1: z = sum_D prior(D) L^u(D) and, for the extrinsic output, zu = sum_D L^u(D)
-    float lu[kFinSym][kFinRegs];
+    float lu[kFinRegs][kFinSym], pr[kFinRegs][kFinSym];
     double z[kFinSym], zu[kFinSym];
-    const bool kept = q <= 32 * kFinRegs;
 #pragma unroll
-    for (int k = 0; k < kFinSym; ++k) {
-        z[k] = zu[k] = 0.0;
+    for (int k = 0; k < kFinSym; ++k) z[k] = zu[k] = 0.0;
+    auto add = [&](int D0, const float (&v)[kFinSym], float (&p)[kFinSym]) {
 #pragma unroll
-        for (int r = 0; r < kFinRegs; ++r) lu[k][r] = 0.f;
-        if (k >= ns) continue;
-        const float *pri = f.priors + (size_t)(i0 + k) * q;
-        if (kept) {
+        for (int k = 0; k < kFinSym; ++k)
+            p[k] = k < ns && D0 + lane < q ? priors[(size_t)(i0 + k) * q + D0 + lane] : 0.f;
 #pragma unroll
-            for (int r = 0; r < kFinRegs; ++r) {
-                const int D = 32 * r + lane;
-                if (32 * r >= q) break;
-                lu[k][r] = lsum(k, D);
-                if (D < q) {
-                    z[k] += (double)pri[D] * (double)lu[k][r];
-                    if (f.ext) zu[k] += (double)lu[k][r];
-                }
-            }
-        } else {
-            for (int D0 = 0; D0 < q; D0 += 32) {
-                const int D = D0 + lane;
-                const float v = lsum(k, D);
-                if (D < q) {
-                    f.app[(size_t)(i0 + k) * q + D] = v;
-                    z[k] += (double)pri[D] * (double)v;
-                    zu[k] += (double)v;
-                }
-            }
+        for (int k = 0; k < kFinSym; ++k) {
+            z[k] += (double)p[k] * (double)v[k];
+            if (ext) zu[k] += (double)v[k];
         }
+    };
+#pragma unroll
+    for (int r = 0; r < kFinRegs; ++r) {
+#pragma unroll
+        for (int k = 0; k < kFinSym; ++k) lu[r][k] = pr[r][k] = 0.f;
+        if (32 * r >= q) continue;
+        lsums(32 * r, lu[r]);
+        add(32 * r, lu[r], pr[r]);
+    }
+    for (int D0 = 32 * kFinRegs; D0 < q; D0 += 32) {  // beyond the registers: through app
+        float v[kFinSym], p[kFinSym];
+        lsums(D0, v);
+        add(D0, v, p);
+#pragma unroll
+        for (int k = 0; k < kFinSym; ++k)
+            if (k < ns && D0 + lane < q) app[(size_t)(i0 + k) * q + D0 + lane] = v[k];
     }
     const double zs = fin_reduce(z, lane);
     const bool ok = mine < ns && zs > 0.0;
     const double iz = ok ? 1.0 / zs : 0.0;
     double izu = 0.0;
-    if (f.ext) {
+    if (ext) {
         const double zus = fin_reduce(zu, lane);
         izu = ok ? 1.0 / zus : 0.0;  // zu >= z / max prior > 0
     }
@@ -646,20 +658,16 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(const FrameDev *__rest
         const double izk = __shfl_sync(0xffffffffu, iz, 4 * k), izuk = __shfl_sync(0xffffffffu, izu, 4 * k);
         if (!(good >> (4 * k) & 1u)) continue;
         const size_t e0 = (size_t)(i0 + k) * q;
-        auto put = [&](int D, float v) {
-            const size_t e = e0 + D;
+        auto put = [&](int D, float p, float v) {
             const double l = (double)v;
-            f.app[e] = (float)((double)f.priors[e] * l * izk);
-            if (f.dpriors) f.dpriors[e] = (float)(l * izk);
-            if (f.ext) f.ext[e] = (float)(l * izuk);
+            app[e0 + D] = (float)((double)p * l * izk);
+            if (dpri) dpri[e0 + D] = (float)(l * izk);
+            if (ext) ext[e0 + D] = (float)(l * izuk);
         };
-        if (kept) {
 #pragma unroll
-            for (int r = 0; r < kFinRegs; ++r)
-                if (32 * r + lane < q) put(32 * r + lane, lu[k][r]);
-        } else {
-            for (int D = lane; D < q; D += 32) put(D, f.app[e0 + D]);
-        }
+        for (int r = 0; r < kFinRegs; ++r)
+            if (32 * r + lane < q) put(32 * r + lane, pr[r][k], lu[r][k]);
+        for (int D = 32 * kFinRegs + lane; D < q; D += 32) put(D, priors[e0 + D], app[e0 + D]);
     }
     if (lane == 0 && good != (ns == kFinSym ? 0xffffffffu : (1u << (4 * ns)) - 1u))
         atomicMax(f.status, ST_ZERO);
@@ -670,19 +678,31 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(const FrameDev *__rest
             const double Pt = f.dPt, Ps = f.dPs, Pd = f.dPd, k = f.kappa;
             const double Qm = k * Pt * (1.0 - Ps), Qs = k * Pt * Ps;
             double Sw = 0.0, Sd = 0.0, Ss = 0.0;
-            float pw = 0.f, pd = 0.f, ps = 0.f;
-            int left = group - (int)((unsigned)tlo % (unsigned)group);
-            for (long long t = tlo; t <= thi; ++t) {
-                const float *gp = f.Gp + row_of(i0 + mine, t) * 3;
-                pw += gp[0];
-                pd += gp[1];
-                ps += gp[2];
-                if (--left == 0 || t == thi) {
-                    Sw += pw;
-                    Sd += pd;
-                    Ss += ps;
-                    pw = pd = ps = 0.f;
-                    left = group;
+            const float *__restrict__ Gp = f.Gp;
+            float sw = 0.f, sd = 0.f, ss = 0.f;
+            int left = (int)(group - (unsigned)tlo % group);
+            for (int t0 = 0; t0 < cnt; t0 += 4) {
+                float x[4][3];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float *g = Gp + row_of(i0 + mine, tlo + min(t0 + e, cnt - 1)) * 3;
+                    x[e][0] = g[0];
+                    x[e][1] = g[1];
+                    x[e][2] = g[2];
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    if (t0 + e >= cnt) break;
+                    sw += x[e][0];
+                    sd += x[e][1];
+                    ss += x[e][2];
+                    if (--left == 0 || t0 + e + 1 == cnt) {
+                        Sw += sw;
+                        Sd += sd;
+                        Ss += ss;
+                        sw = sd = ss = 0.f;
+                        left = (int)group;
+                    }
                 }
             }
             // Sw, Sd, Ss: sums with dR~/dw', dR~/dPd, dR~/dQ's.  R~ is homogeneous
