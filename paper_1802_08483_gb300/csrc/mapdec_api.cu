@@ -214,6 +214,7 @@ struct FrameHost {
     bool tc = false;        // forward producer on the tensor cores
     bool tcb = false;       // APP producer on the tensor cores
     bool split = false;     // APP super-tiles may be shortened to fill the GPU
+    bool fit = false;       // and tiles
     std::vector<float> phi0, phiN;  // boundary drift priors (stream decoding), or empty
     int64_t phi_off = 0;    // float offset of phi0 (then phiN) in the batch's buffer
 };
@@ -579,6 +580,48 @@ size_t frame_scratch_floats_seg(const FrameDev &f, int K, int S, bool grad) {
     return s;
 }
 
+// Tiles of the CUDA-core producers for a launch of `positions` received positions
+// in all (the frames at their largest received length).  W does not depend on the
+// forward tile, so it is chosen by itself: a gradient frame's APP tile is short
+// (four metrics per position), and a forward producer on it leaves a third of
+// its threads without a lattice and reloads the priors for every few positions; it takes up to
+// 1024 lattices (four rounds of the CTA) in half the shared-memory budget.  With
+// fewer than two CTAs per SM, tiles are halved down to one round of lattices; in
+// decode mode the APP producer's too.
+// Whole passes: 48 gradient frames N = 2000, q = 32 39.1 -> 35.6 ms; one frame
+// N = 50, q = 16 184 -> 171 us, N = 300, q = 32 406 -> 378 us.
+void fit_fwd_tile(FrameDev &f, long long positions, bool grad) {
+    const int sms = device_sms() > 0 ? device_sms() : 152;
+    auto span = [&](int c) { return (int)((c - 1 + 2LL * f.xmax) / f.n + 2); };
+    int c = f.P;
+    if (grad) {
+        for (int d : {64, 48, 32, 24, 16, 12, 8}) {
+            FrameDev t = f;
+            t.Pf = d;
+            t.Sf = span(d);
+            if (d > c && d * f.q <= 1024 && fwd_smem_bytes(t) <= kFwdSmemBudget / 2) {
+                c = d;
+                break;
+            }
+        }
+    }
+    while (c > 1 && (long long)c * f.q > kThreads && positions / c < 2LL * sms) c /= 2;
+    f.Pf = c;
+    f.Sf = span(c);
+    f.Tf = (int)((f.rho + 1 + c - 1) / c);
+}
+void fit_app_tile(FrameDev &f, long long positions) {
+    const int sms = device_sms() > 0 ? device_sms() : 152;
+    int c = f.P;
+    while (c > 1 && (long long)c * f.q > kThreads && positions / c < 2LL * sms) c /= 2;
+    if (c == f.P) return;
+    f.P = c;
+    f.S = (int)((c - 1 + 2LL * f.xmax) / f.n + 2);
+    f.nsub = 1;
+    f.S2 = f.S;
+    f.T = f.T2 = (int)((f.rho + 1 + c - 1) / c);
+}
+
 // APP super-tiles short enough for a launch to fill the GPU.  plan_shape's
 // super-tiles of 256 positions amortise a CTA's set-up over a large batch, but a
 // single frame or a checkpointed batch's segment is then a handful of CTAs on 152
@@ -852,7 +895,8 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
     b->grad = (flags & MAPDEC_BATCH_GRAD) != 0;
     b->segmented = (flags & MAPDEC_BATCH_SEGMENTED) != 0;
     b->fr.resize(nf);
-    std::map<std::pair<int, int>, long long> class_ctas;  // APP-producer CTAs per (n, I) launch
+    // per (n, I) launch: APP-producer CTAs, received positions
+    std::map<std::pair<int, int>, long long> class_ctas, class_pos;
     for (int i = 0; i < nf; ++i) {
         FrameHost &h = b->fr[i];
         h.d = frames[i];
@@ -979,6 +1023,9 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
         }
         h.split = !b->grad && !per_sym && !h.tcb && !(tuned && tu.nsub > 0) &&
                   !std::getenv("MAPDEC_FORCE_NSUB");
+        class_pos[{h.d.n, h.d.I}] += b->segmented ? (long long)h.d.n * h.segK + 2LL * h.d.xmax
+                                                  : (long long)h.d.n * h.d.N + h.d.xmax + 1;
+        h.fit = !per_sym && !h.store && !(tuned && tu.P > 0) && (plain || forceP <= 0);
         if (b->grad && !per_sym) {
             // partial sums per sub-tile; the order of the sums stays that of the
             // planned super-tiles
@@ -1002,6 +1049,9 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
         b->phi_total += (int64_t)(h.phi0.size() + h.phiN.size());
     }
     for (auto &h : b->fr) {
+        const long long pos = class_pos[{h.d.n, h.d.I}];
+        if (h.fit && h.split) fit_app_tile(h.dev, pos);
+        if (h.fit && !h.tc) fit_fwd_tile(h.dev, pos, b->grad);
         if (h.split) split_supertiles(h.dev, supertile_split(class_ctas[{h.d.n, h.d.I}]));
         if (h.dev.group) {  // eight CTAs per SM, no more sub-tiles each than planned
             const int sms = device_sms() > 0 ? device_sms() : 152;
@@ -2104,7 +2154,10 @@ int mapdec_decode_noalloc(const mapdec_frame_desc_t *frame, const uint8_t *rx_de
 
     FrameDev f{};
     plan_shape(f, d, false, 0);
+    const long long pos = (long long)f.n * f.N + f.xmax + 1;
     split_supertiles(f, supertile_split(most_supertiles(f)));
+    fit_app_tile(f, pos);
+    fit_fwd_tile(f, pos, false);
     const int cl = chain_cluster(2, f.chainNV);
     const int cthr = chain_threads(cl, f.chainVWarps, f.chainNV);
     plan_chain(f, cl, cthr, chain_ask(nullptr));

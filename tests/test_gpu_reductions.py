@@ -63,6 +63,25 @@ def test_long_codewords(n, I):
     check_ll(ll[0], ll_ref)
 
 
+# lone frames whose tiles are cut to one round of lattices: q that divides the
+# 256 threads or not, one that fills a round alone
+@pytest.mark.parametrize("q,n", [(3, 4), (48, 6), (64, 7), (256, 9)])
+def test_short_tiles(q, n):
+    N, xmax = 25, 20
+    fr = synth.make_frame(np.random.default_rng(q), q, n, N, 2, xmax, 0.04, 0.04, 0.01, dirichlet=True)
+    ref, ll_ref = oracle.decode(fr.codebook, N, 0.04, 0.04, 0.01, 2, xmax, fr.rx, priors=fr.priors,
+                                kappa=2.0)
+    dec = mapdec.Decoder.for_frame(fr)
+    app, ll = dec.decode(fr.rx, fr.priors)
+    llg, dchan, _ = dec.loglik_grad(fr.rx, fr.priors)
+    dec.close()
+    check_app(app, ref)
+    check_ll(ll, ll_ref)
+    check_ll(llg, ll_ref)
+    check_grad(dchan, oracle.loglik_grad(fr.codebook, N, 0.04, 0.04, 0.01, 2, xmax, fr.rx,
+                                         priors=fr.priors)[1])
+
+
 def test_many_supertiles_per_symbol():
     """A lone frame's super-tiles are short: a symbol's window spans more than the
     32 partial rows that finalize looks up at a time."""
