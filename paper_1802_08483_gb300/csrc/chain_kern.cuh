@@ -325,6 +325,12 @@ struct WeightTab {
 // 420 us; gradients of N = 1000, M = 121, MN = 25: 2.36 -> 1.48 ms; 64 stream frames
 // N = 1000, M = 171: 4.66 -> 3.68 ms; 8 frames N = 8000, M = 1661, MN = 49,
 // checkpointed: 287 -> 208 ms.
+// Bookkeeping that every warp repeats is kept to one step counter, and what only
+// the storer needs to shared memory (with more live values the 512-thread modes
+// spill, and a cluster barrier waits for the spills' stores: 1.45 -> 1.61 ms).
+// Recursions alone, with a counter per quantity and so: N = 50, M = 41 99.9 -> 91.7
+// us; N = 300, M = 81 298 -> 282; N = 1000, M = 121 861 -> 803; N = 1000, M = 401
+// 1481 -> 1447; 64 stream frames M = 171 1141 -> 1070.
 template <int MNT, int MODE>
 __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kChainMaxThreads) k_chain(
     const FrameDev *__restrict__ frames, const Work *__restrict__ work) {
@@ -512,8 +518,8 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
             else rows[s] = (dir == 0) ? f.ckpt[s] : f.bedge[s];
         }
     }
-    float *grow = (dir == 0) ? f.alpha + (size_t)i0 * Mp : f.beta + (size_t)i1 * Mp;
-    const long long gstep = dir == 0 ? Mp : -Mp;
+    float *const grow = (dir == 0) ? f.alpha + (size_t)i0 * Mp : f.beta + (size_t)i1 * Mp;
+    const long long gstep = dir == 0 ? Mp : -Mp;  // row t of this launch: grow + t gstep
     if (rank == 0)
         for (int s = tid; s < M; s += nthr) grow[s] = rows[s];  // this thread's own entries
 
@@ -523,7 +529,7 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
     float lrow = 0.f;     // log2 of the current row's sum
     float lc_prev = 0.f;  // sum of log2 growth since the last tilt update
     int lc_cnt = 0;       // number of steps in lc_prev
-    int steps = 0;        // steps taken in this direction so far
+    int steps0 = 0;       // steps of this direction before this launch
     double ztilt = 0.0;
     if (!fresh && segm && !replay) {
         const ChainState &cs = f.cst[dir];
@@ -532,7 +538,7 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
         lc_prev = cs.lc_sum;
         lrow = cs.lrow;
         lc_cnt = cs.lc_cnt;
-        steps = cs.steps;
+        steps0 = cs.steps;
         zexp = (int)cs.zexp;
         ztilt = cs.ztilt;
     }
@@ -573,7 +579,8 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
     // Sums of the rows built since the last time (pend of them), in the order of
     // 256 virtual lanes: partial sums and first moments x[2 k], x[2 k + 1] of this
     // lane (k = 3 the last row), butterflies into s_red[.][virtual warp].
-    int pend = 0, cb = 0;  // cb: ring buffer of the last row
+    int pend = 0, cur = 0;  // cur: the last row's buffer in the ring (floats)
+    const int rowE = RB * RS;
     const int CD = f.chainCD, nwi = f.chainVWarps;
     float x[8];
 #pragma unroll
@@ -617,13 +624,13 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
                 for (int l = wi * 32 + lane; l < (nst << lg); l += 256) {
                     const int s = s00 + (l >> lg);
                     const float m = (float)(s - xmax);
-                    int q = cb;
+                    int q = cur;
 #pragma unroll
                     for (int k = 3; k >= 0; --k) {
-                        const float v = (l & js) || k < 4 - pend ? 0.f : rows[q * RS + s];
+                        const float v = (l & js) || k < 4 - pend ? 0.f : rows[q + s];
                         x[2 * k] += v;
                         x[2 * k + 1] = fmaf(v, m, x[2 * k + 1]);
-                        q = q == 0 ? RB - 1 : q - 1;
+                        q = q == 0 ? rowE - RS : q - RS;
                     }
                 }
             }
@@ -635,10 +642,11 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
     float sc_last = 1.f;            // scales the last summed row
     int rec_row = -1;               // mover: a row whose mean is to be recorded
     float rec_mean = 0.f;
-    float qs0 = 0.f, qs1 = 0.f, qs2 = 0.f, qs3 = 0.f;  // storer: scales of the rows to store, in order
-    int qn = 0, qb = 0;             // how many, ring buffer of the first
-    float *qg = grow;               // and its place
-    auto sum_rows = [&](int row_last) -> bool {
+    __shared__ float s_qs[4];       // storer: scales of the rows to store, the last in entry 3
+    int qn = 0, qb = 0;             // how many, buffer of the first
+    int qr = 0;                     // and its row number
+    // st: the row number of the last one in this launch
+    auto sum_rows = [&](int st) -> bool {
         bool good;
         float mn;
         if (pend == 1) {
@@ -657,8 +665,8 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
             lrow = l - (float)e;
             zexp += e;
             sc_last = inv_pow2(e);
-            qs0 = sc_last;
-            if (record && dir == 0 && mover && lane == 0) { rec_row = row_last; rec_mean = mn; }
+            if (storer && lane == 0) s_qs[3] = sc_last;
+            if (record && dir == 0 && mover && lane == 0) { rec_row = i0 + st; rec_mean = mn; }
         } else {
             // lane 2 k: sum c of row k; lane 2 k + 1: its first moment
             const float4 ra = *reinterpret_cast<const float4 *>(&s_red[lane & 7][0]);
@@ -677,7 +685,7 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
             good = (ok & ((0x55u << (2 * k0)) & 0x55u)) == ((0x55u << (2 * k0)) & 0x55u);
             const int row = (lane >> 1) - k0;  // rows since the last time
             if (record && dir == 0 && mover && lane < 8 && !(lane & 1) && row >= 0) {
-                rec_row = row_last - (pend - 1 - row);
+                rec_row = i0 + st - (pend - 1 - row);
                 rec_mean = mn;
             }
             const int eo = e - dp;
@@ -694,30 +702,29 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
             mn = __shfl_sync(0xffffffffu, mn, 6);
             const float sc = inv_pow2(e);
             sc_last = __shfl_sync(0xffffffffu, sc, 6);
-            if (storer) {
-                qs0 = __shfl_sync(0xffffffffu, sc, 2 * k0);
-                qs1 = __shfl_sync(0xffffffffu, sc, min(6, 2 * k0 + 2));
-                qs2 = __shfl_sync(0xffffffffu, sc, min(6, 2 * k0 + 4));
-                qs3 = sc_last;
-            }
+            if (storer && lane < 8 && !(lane & 1)) s_qs[lane >> 1] = sc;
         }
         lc_cnt += pend;
         mean = mn;
-        qn = pend;
-        qb = cb - (pend - 1);
-        if (qb < 0) qb += RB;
-        qg = grow - (pend - 1) * gstep;
+        if (storer) {
+            qn = pend;
+            qb = cur - (pend - 1) * RS;
+            if (qb < 0) qb += rowE;
+            qr = st - (pend - 1);
+            __syncwarp();
+        }
         pend = 0;
         return good;
     };
     // The storer writes a summed row, scaled, to global memory: one a step.
     auto store_row = [&]() {
         if (qn == 0) return;
-        const float *r = rows + qb * RS;
-        for (int s = rank * 32 + lane; s < M; s += 32 * ncta) qg[s] = r[s] * qs0;
-        qs0 = qs1; qs1 = qs2; qs2 = qs3;
-        qg += gstep;
-        qb = qb + 1 == RB ? 0 : qb + 1;
+        const float *r = rows + qb;
+        const float sc = s_qs[4 - qn];
+        float *const g = grow + qr * gstep;
+        for (int s = rank * 32 + lane; s < M; s += 32 * ncta) g[s] = r[s] * sc;
+        ++qr;
+        qb = qb + RS == rowE ? 0 : qb + RS;
         --qn;
     };
 
@@ -780,22 +787,26 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
     bool failed = false, alive = true, ready = false;
     const int cap = f.chainCap;
     const bool inplace = f.chainRing == 2;
-    // places in floats: stage, row buffer, weight table
-    int slot = 0, cur = 0;
-    const int slotB = (int)stageFloats, slotE = NST * slotB, rowE = RB * RS;
+    int slot = 0;  // the coming chunk's stage (floats)
+    const int slotB = (int)stageFloats, slotE = NST * slotB;
     const int off0 = vB > vA ? tab[0].off : 0;
     const float *const wts = wtab[0].plain;
     constexpr int kWt = sizeof(WeightTab) / 4;
+    // the steps [q0, q1) with every W row valid, in a CTA whose warps have one
+    // lane group each: a loop of their own
+    int q0 = nsteps, q1 = nsteps;
+    if (nck == 1 && LL <= 2) {
+        q0 = max(0, dir == 0 ? iin0 - i0 : i1 - 1 - iin1);
+        q1 = min(nsteps, dir == 0 ? iin1 - i0 + 1 : i1 - iin0);
+    }
     chain_sync<CL>();  // rows, first chunk ready in every CTA
     int st = 0;
     while (st < nsteps) {
-        int i = dir == 0 ? i0 + st : i1 - 1 - st;
-        if (s_fail) {
-            failed = true;
-            break;
-        }
+        const int steps = steps0 + st;
+        const int gave_up = s_fail;
         const bool due = replay || tilt_due(steps);
         const bool summed = pend > 0 && (ready || !alive);
+        bool good = true;
         if (summed) {
             if (storer)
                 while (qn > 0) store_row();
@@ -806,11 +817,12 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
                 if (!helper && has) reduce_rows(warp);
                 __syncthreads();
             }
-            if (!sum_rows(dir == 0 ? i : i + 1)) {
-                failed = true;
-                break;
-            }
+            good = sum_rows(st);
             alive = true;
+        }
+        if (gave_up || !good) {
+            failed = true;
+            break;
         }
         // tilt of the new row (the recompute sweep replays the recorded ones)
         float tn = theta;
@@ -818,8 +830,8 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
             tn = th_next;
             mean = mc_next;
             if (st + 1 < nsteps) {
-                th_next = (float)thr_[i + 2];
-                mc_next = (float)mcr[i + 1];
+                th_next = (float)thr_[i0 + st + 2];
+                mc_next = (float)mcr[i0 + st + 1];
             }
         } else if (due) {
             if (steps > 0 && lc_cnt > 0) {
@@ -836,25 +848,24 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
         }
         float dth = dir == 0 ? tn - theta : theta - tn;
         // the row's power of two, and forward its change of tilt (backward: on
-        // the new row), into the next buffer: the mover stores the row as it was
+        // the new row), into the next buffer: the storer writes the row as it was
         const bool pre = dir == 0 && dth != 0.f;
+        int wt = vp * kWt;
         if (summed || pre) {
             const float sc = summed ? sc_last : 1.f;
             int to = cur + RS == rowE ? 0 : cur + RS;
             if (inplace) to = cur;
             for (int s = tid; s < M; s += nthr) {
                 float v = rows[cur + s] * sc;
-                if (inplace && summed && rank == 0) grow[s] = v;
+                if (inplace && summed && rank == 0) grow[st * gstep + s] = v;
                 if (pre) v *= exp2f(dth * ((float)(s - xmax) - mean));
                 rows[to + s] = v;
             }
             if (inplace) qn = 0;
-            else cb = cb + 1 == RB ? 0 : cb + 1;
             cur = to;
         }
         // weights 2^{(theta - 1) j}: forward of the new tilt, backward of the
         // source row's (the other table, from the next step on)
-        int wt = vp * kWt;
         if (tn != th_tab) {
             if (dir == 1) vp ^= 1;
             fill_weights(wtab[vp], tn);
@@ -863,25 +874,25 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
         if (summed || pre) __syncthreads();
         // FP64 records by the mover, while the others compute
         if (mover) {
-            if (dir == 0 && tn != theta) ztilt += (double)(tn - theta) * ((double)n * i + (double)mean);
+            if (dir == 0 && tn != theta)
+                ztilt += (double)(tn - theta) * ((double)n * (i0 + st) + (double)mean);
             if (rec_row >= 0) mcr[rec_row] = (double)rec_mean;
             rec_row = -1;
         }
-        // steps until the rows are summed again
+        theta = tn;
+        // steps until the rows are summed again, at the last of them unless the
+        // recompute sweep needs no sums there
         const int run = replay || steps < kTiltSettle
                             ? 1
                             : min(min(nsteps - st, cap - pend), kTiltEvery - (steps & (kTiltEvery - 1)));
-        // plain steps of a warp with one lane group: a loop of its own, with the
-        // kind of its sums fixed at compile time
-        int quick = 0;
-        if (nck == 1 && LL <= 2 && i >= iin0 && i <= iin1)
-            quick = min(run, dir == 0 ? iin1 - i + 1 : i - iin0 + 1);
+        const bool sums = !replay || st + 1 == nsteps || pend + 1 == cap || th_next != tn;
+        const int quick = st >= q0 ? min(run, q1 - st) : 0;
+        int done = 0;
         if (quick > 0) {
-            // the last of them sums its rows where the next tilt update needs them
-            const bool fin = quick == run && (!replay || st + 1 == nsteps || pend + 1 == cap || th_next != tn);
+            const bool fin = sums && quick == run;
             int u = 0;
             if (mover) {
-                double *tr = thr_ + (dir == 0 ? i + 1 : i);
+                double *tr = thr_ + (dir == 0 ? i0 + st + 1 : i1 - 1 - st);
                 const double tnd = (double)tn;
                 for (;;) {
                     if (record && lane == 0) *tr = tnd;
@@ -936,24 +947,26 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
                     }
                 });
             }
-            dth = 0.f;
-            wt = vp * kWt;
             ready = fin && u == quick;
+            done = u;
             pend += u;
-            steps += u;
-            st += u;
-            i += dir == 0 ? u : -u;
-            grow += u * gstep;
-            cb += u;
-            if (cb >= RB) cb -= RB;
-            cur = cb * RS;
-            for (int k = 0; k < u; ++k) slot = slot + slotB == slotE ? 0 : slot + slotB;
+            cur += u * RS;
+            if (cur >= rowE) cur -= rowE;
+            slot += u * slotB;
+            if (slot >= slotE) slot -= slotE;
+            if (slot >= slotE) slot %= slotE;  // fewer stages than steps in a run
         }
-        for (int u = quick; u < run && alive; ++u) {
+        st += done;
+        for (int u = done; u < run && alive; ++u, ++st) {
+            const int i = dir == 0 ? i0 + st : i1 - 1 - st;
+            if (u > 0) {
+                wt = vp * kWt;
+                dth = 0.f;
+            }
             const bool inner = i >= iin0 && i <= iin1;
             const int nxt = cur + RS == rowE ? 0 : cur + RS;
             ++pend;
-            ready = u + 1 == run && (!replay || st + 1 == nsteps || pend == cap || th_next != tn);
+            ready = u + 1 == run && sums;
             bool some = false;
             if (mover) {
                 if (record && lane == 0) thr_[dir == 0 ? i + 1 : i] = (double)tn;
@@ -1019,15 +1032,7 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
             if (mover && issued < total) issue_next();
             for (int k = 0; k < nck; ++k) slot = slot + slotB == slotE ? 0 : slot + slotB;
             cur = nxt;
-            cb = cb + 1 == RB ? 0 : cb + 1;
-            grow += gstep;
-            ++steps;
-            ++st;
-            i += dir == 0 ? 1 : -1;
-            wt = vp * kWt;
-            dth = 0.f;
         }
-        theta = tn;
     }
     if (!failed && s_fail) failed = true;
     if (!failed && pend > 0) {  // the last rows (the last step's sums are ready)
@@ -1037,7 +1042,7 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
             gather_rows();
             __syncthreads();
         }
-        failed = !sum_rows(dir == 0 ? i1 : i0);
+        failed = !sum_rows(nsteps);
         if (storer)
             while (qn > 0) store_row();
         if (mover && rec_row >= 0) mcr[rec_row] = (double)rec_mean;
@@ -1052,7 +1057,7 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
         __syncthreads();
         return;
     }
-    const float *last = rows + cb * RS;
+    const float *last = rows + cur;
     const float inv = sc_last;
     if (segm && !replay) {
         // carry the boundary row and the controller state to the next launch
@@ -1066,7 +1071,7 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
             cs.lc_sum = lc_prev;
             cs.lrow = lrow;
             cs.lc_cnt = lc_cnt;
-            cs.steps = steps;
+            cs.steps = steps0 + nsteps;
             cs.zexp = zexp;
             cs.ztilt = ztilt;
         }
