@@ -28,6 +28,19 @@ __device__ __forceinline__ int ps_group_lanes(int q) {
     return g;
 }
 
+// CTAs per SM asked of the compiler (0: its own choice).  Held to 128 registers two
+// CTAs are resident instead of one, which hides the lattices' latency; with few
+// values the kernel needs no more, with many the spills cost more than they give.
+// 16 frames N = 600, phase times at one CTA and two: forward MN = 13 187 -> 172 us
+// (MN = 10: 82 -> 90), 25 475 -> 379, 31 (xmax 85) 1655 -> 1456, 41 1694 -> 1544
+// (MN = 49: 3436 -> 3457); backward MN = 31 892 -> 684, 37 3504 -> 3062, 49 1423 ->
+// 1214 (MN = 28: 934 -> 989, 25: 269 -> 280).  All of these include the lattices'
+// shorter tails (eval_metric_x).
+constexpr int ps_fwd_ctas(int NB, int IB) {
+    return NB * (IB + 1) + 1 >= 13 && NB * (IB + 1) + 1 <= 41 ? 2 : 0;
+}
+constexpr int ps_bwd_ctas(int NB, int IB) { return NB * (IB + 1) + 1 >= 31 ? 2 : 0; }
+
 // Lattice (p, x) with an explicit codeword; out[j] for j < MN, zero past rho.
 template <int NB, int IB, int MODE>
 __device__ __forceinline__ void eval_metric_x(const FrameDev &f, long long p, uint32_t x,
@@ -36,13 +49,14 @@ __device__ __forceinline__ void eval_metric_x(const FrameDev &f, long long p, ui
     float F[kMaxMN], T[kMaxMN];
     const uint64_t y = rx_window(f.rxbits, p);
     lattice_any<NB, IB, MODE>(f, x, y, F, T);
-    const long long lim = f.rho - p;
 #pragma unroll
-    for (int j = 0; j < ((NB == 0) ? kMaxMN : NB * (IB + 1) + 1); ++j) {
-        if (j < MN) {
-            const float v = MODE ? T[j] : F[j];
-            out[j] = (j <= lim) ? v : 0.f;
-        }
+    for (int j = 0; j < ((NB == 0) ? kMaxMN : NB * (IB + 1) + 1); ++j)
+        if (j < MN) out[j] = MODE ? T[j] : F[j];
+    const long long lim = f.rho - p;
+    if (lim < MN - 1) {  // the frame's last positions only
+#pragma unroll
+        for (int j = 0; j < ((NB == 0) ? kMaxMN : NB * (IB + 1) + 1); ++j)
+            if (j < MN && j > lim) out[j] = 0.f;
     }
 }
 
@@ -52,7 +66,8 @@ __device__ __forceinline__ void eval_metric_x(const FrameDev &f, long long p, ui
 // butterfly per value took MN log2 G of each, and neighbouring lanes store
 // neighbouring values.  The additions and their order per value are the same.
 // 16 frames (N = 1000, q = 16, n = 10, I = 2, xmax = 85): the whole decode 9.74 ms
-// with a butterfly per value, 6.25 ms with this; bound by the lattices since.
+// with a butterfly per value, 6.25 ms with this.  Bound by the lattices since (70% of
+// issue slots; selects on the ALU pipe and FMAs in equal parts).
 template <int MNC, int G>
 __device__ __forceinline__ void ps_reduce_store(const float (&acc)[MNC], int gl, int MN, bool store,
                                                 float *row) {
@@ -81,7 +96,7 @@ __device__ __forceinline__ void ps_reduce_store(const float (&acc)[MNC], int gl,
 }
 
 template <int NB, int IB>
-__global__ void __launch_bounds__(kThreads) k_fwd_ps(const FrameDev *__restrict__ frames,
+__global__ void __launch_bounds__(kThreads, ps_fwd_ctas(NB, IB)) k_fwd_ps(const FrameDev *__restrict__ frames,
                                                      const Work *__restrict__ work) {
     const Work wk = work[blockIdx.x];
     const FrameDev &f = frames[wk.frame];
@@ -129,7 +144,7 @@ __global__ void __launch_bounds__(kThreads) k_fwd_ps(const FrameDev *__restrict_
 // smem: Aw[psC][4], Bw[psC + MN - 1][4] (the windows of one symbol, row
 // stride 4), 4 x 4 tilt constants, red[ngrp][q][NR] (per-group sums).
 template <int NB, int IB, bool GRAD>
-__global__ void __launch_bounds__(kThreads) k_bwd_ps(const FrameDev *__restrict__ frames,
+__global__ void __launch_bounds__(kThreads, GRAD ? 0 : ps_bwd_ctas(NB, IB)) k_bwd_ps(const FrameDev *__restrict__ frames,
                                                      const Work *__restrict__ work) {
     constexpr int NR = GRAD ? 4 : 1;
     const Work wk = work[blockIdx.x];
