@@ -330,7 +330,8 @@ struct WeightTab {
 // spill, and a cluster barrier waits for the spills' stores: 1.45 -> 1.61 ms).
 // Recursions alone, with a counter per quantity and so: N = 50, M = 41 99.9 -> 91.7
 // us; N = 300, M = 81 298 -> 282; N = 1000, M = 121 861 -> 803; N = 1000, M = 401
-// 1481 -> 1447; 64 stream frames M = 171 1141 -> 1070.
+// 1481 -> 1447; 64 stream frames M = 171 1141 -> 1070; against it the whole decode of
+// the 8 frames N = 8000, M = 1661 (several lane groups a warp) 198.9 -> 200.4 ms.
 template <int MNT, int MODE>
 __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kChainMaxThreads) k_chain(
     const FrameDev *__restrict__ frames, const Work *__restrict__ work) {

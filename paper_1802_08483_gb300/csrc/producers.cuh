@@ -42,8 +42,9 @@ __device__ __forceinline__ void lattice_any(const FrameDev &f, uint32_t x, uint6
 // frame's last positions have such j, so it is one branch (a 64-bit compare and a
 // select per value took up to a tenth of a lattice's instructions; 64 stream frames
 // N = 1000, q = 16, n = 10: k_fwd 1092 -> 1053 us, k_bwd 1265 -> 1232 us; 48 gradient
-// frames N = 2000, q = 32, n = 8, whole pass 35.5 -> 34.3 ms; against it 8 frames
-// N = 8000, q = 64, n = 12, I = 3, more spills there: 198.8 -> 200.4 ms).
+// frames N = 2000, q = 32, n = 8, whole pass 35.5 -> 34.3 ms; 16 frames N = 150,
+// n = 15 892 -> 864 us; 8 frames N = 8000, n = 12, I = 3 200.4 -> 200.7 ms, where the
+// values' count is large and the branch gives nothing).
 // MODE 0 -> R; MODE k > 0 -> the k-th tangent.
 template <int NB, int IB, int MODE>
 __device__ __forceinline__ void eval_metric(const FrameDev &f, long long p, int D, float *out) {
