@@ -1025,7 +1025,8 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
                   !std::getenv("MAPDEC_FORCE_NSUB");
         class_pos[{h.d.n, h.d.I}] += b->segmented ? (long long)h.d.n * h.segK + 2LL * h.d.xmax
                                                   : (long long)h.d.n * h.d.N + h.d.xmax + 1;
-        h.fit = !per_sym && !h.store && !(tuned && tu.P > 0) && (plain || forceP <= 0);
+        // stored metrics: both producers on one tile, so only where both are fitted
+        h.fit = !per_sym && (!h.store || h.split) && !(tuned && tu.P > 0) && (plain || forceP <= 0);
         if (b->grad && !per_sym) {
             // partial sums per sub-tile; the order of the sums stays that of the
             // planned super-tiles
