@@ -307,11 +307,11 @@ __device__ __forceinline__ void window_tilt(int S, int S4, int P, int BW, float 
 // ---------------------------------------------------------------------------
 // Backward producer (APP partial sums, optional tangents).  One CTA owns a
 // super-tile of nsub sub-tiles of P positions and accumulates, in shared
-// memory, for every symbol i it touches (gradient mode: stores for every
-// sub-tile, so that the CTAs can be short enough to fill the GPU while finalize
-// adds the sub-tiles up in one fixed order; 48 frames N = 2000, q = 32, segments of
-// 45 symbols: super-tiles of 42 sub-tiles were 144 CTAs a launch, the whole pass
-// 67.4 ms; of 3 sub-tiles 41.3 ms):
+// memory, for every symbol i it touches (frames planned for gradients, f.group > 0,
+// in decode calls too: stores for every sub-tile, so that the CTAs can be short
+// enough to fill the GPU while finalize adds the sub-tiles up in one fixed order;
+// 48 frames N = 2000, q = 32, segments of 45 symbols: super-tiles of 42 sub-tiles
+// were 144 CTAs a launch, the whole pass 67.4 ms; of 3 sub-tiles 41.3 ms):
 //   Lacc[i][D] = sum_{p in super-tile, j} alpha_i(s') R[p][D][j] beta_{i+1}(s'+j-n)
 //   Gacc[i][t] = sum_D prior_i(D) (the same sum with the t-th tangent of R)
 // Per sub-tile the contraction is evaluated as
@@ -352,8 +352,9 @@ __global__ void __launch_bounds__(kThreads, (GRAD && (NB == 0 || NB > 10)) ? 1 :
     float *symPhi = symG + Smax4;                               // theta'_{i+1} - 1
     float *Lacc = symPhi + Smax4;
     float *Ct = Lacc;  // gradient mode (no accumulators)
+    const bool apart = GRAD || f.group != 0;  // rows of Lp per sub-tile
 
-    if (!GRAD)
+    if (!apart)
         for (int idx = threadIdx.x; idx < S2 * q; idx += blockDim.x) Lacc[idx] = 0.f;
 
     for (int sub = 0; sub < f.nsub; ++sub) {
@@ -365,7 +366,7 @@ __global__ void __launch_bounds__(kThreads, (GRAD && (NB == 0 || NB > 10)) ? 1 :
         if (S <= 0) continue;
         const int S4 = (S + 3) & ~3;
         const int off = ilo - ilo2;  // row of symbol ilo in the accumulators
-        // gradient mode: the sub-tile's rows of Lp and Gp
+        // the sub-tile's rows of Lp and Gp
         const size_t row0 = (size_t)((long long)wk.tile * f.nsub + sub) * f.S2;
 
         // (B) alpha and beta windows of the sub-tile's symbols (see
@@ -486,7 +487,7 @@ __global__ void __launch_bounds__(kThreads, (GRAD && (NB == 0 || NB > 10)) ? 1 :
                         const int th = col / DS, D = col - th * DS;
                         if (D >= q) continue;
                         if (th == 0) {
-                            if (GRAD) f.Lp[(row0 + il) * q + D] = acc[r][c];
+                            if (apart) f.Lp[(row0 + il) * q + D] = acc[r][c];
                             else Lacc[(size_t)(off + il) * q + D] += acc[r][c];
                         } else Ct[((size_t)(th - 1) * Smax4 + il) * DS + D] = acc[r][c];
                     }
@@ -506,7 +507,7 @@ __global__ void __launch_bounds__(kThreads, (GRAD && (NB == 0 || NB > 10)) ? 1 :
         }
         __syncthreads();
     }
-    if (GRAD) return;
+    if (apart) return;
     const size_t row0 = (size_t)wk.tile * f.S2;
     for (int idx = threadIdx.x; idx < S2 * q; idx += blockDim.x)
         f.Lp[row0 * q + idx] = Lacc[idx];
