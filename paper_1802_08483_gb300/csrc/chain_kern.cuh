@@ -27,6 +27,8 @@ constexpr int kTiltSettle = 64;  // updates every step for the first steps
 // Rows are divided by their power of two when their sums are formed (at tilt
 // updates), or at once when their largest entry fell below this.
 constexpr float kRowLow = 1.f / 65536.f;
+constexpr int kRunMost = 4;      // rows between two sums, at most
+constexpr int kAliveSlots = 16;  // steps until a vote's place is used again (a power of two)
 
 __device__ __forceinline__ bool tilt_due(int steps) {
     return steps < kTiltSettle || (steps & (kTiltEvery - 1)) == 0;
@@ -49,19 +51,29 @@ __device__ __forceinline__ void st_cluster(const void *p, uint32_t rank, uint32_
     asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 // Barrier over the recursion's CTAs (one, or the cluster).
-// helper: a warp whose stores (to global memory) no CTA of the cluster reads, so
-// that its arrival need not wait for them.
+// relaxed (the helper warps of a cluster): the arrival orders nothing by itself, so
+// it need not wait for the warp's earlier stores.  The storer's all go to global
+// memory and are read by no CTA of the launch (waiting for a row's took about 1000
+// clocks).  The mover hands the landed W on to its own CTA, by a fence of that scope
+// (cta_release).  The compute warps' arrivals release rows and votes to the cluster.
+// What a helper reads (rows, votes) is ordered before later writes of other warps by
+// the CTA's barriers (__syncthreads) at the sums, one in four steps at least, and the
+// compute warps' releases after them: the ring of rows and the votes' places are long
+// enough for that.
 template <bool CL>
-__device__ __forceinline__ void chain_sync(bool helper = false) {
+__device__ __forceinline__ void chain_sync(bool relaxed = false) {
     if constexpr (CL) {
         __syncwarp();
-        if (helper) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+        if (relaxed) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
         else asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     } else {
         __syncthreads();
     }
 }
+
+// Orders what this warp saw or wrote before its relaxed arrival, for its own CTA.
+__device__ __forceinline__ void cta_release() { asm volatile("fence.acq_rel.cta;" ::: "memory"); }
 
 // A lane group: 32 consecutive lanes of one chunk of states, JS = 2^lg adjacent
 // lanes per state (state = s0 + (lane >> lg), below d1).
@@ -312,7 +324,8 @@ struct WeightTab {
 //     of W_i (cp.async.bulk on mbarriers, every wait bounded, several steps
 //     ahead), waits for the next step's before it joins the step's barrier, and
 //     writes the tilts and the FP64 record; the storer writes the summed rows,
-//     scaled, to global memory, one a step.
+//     scaled, to global memory, one a step (and in a cluster the tilts and means,
+//     see chain_sync).
 //   - A row of many states takes a warp per lane group, and, with SMs idle, the
 //     CTAs of a cluster: each stages its part of W_i (one SM streams 64 bytes a
 //     clock) and stores its states into every CTA's row buffers through
@@ -362,7 +375,7 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
     const int nck = max(1, (vB - vA + CK - 1) / CK);  // a CTA without states steps along
 
     __shared__ uint64_t bar[kMaxStages];
-    __shared__ int s_alive[4];  // clusters, by step & 3: some entry >= kRowLow
+    __shared__ int s_alive[kAliveSlots];  // clusters, by step: some entry >= kRowLow
     __shared__ int s_fail;      // status of a wait that gave up
     __shared__ __align__(16) float s_red[8][8];   // [2 row + (sum, moment)][virtual warp]
     __shared__ __align__(16) WeightTab wtab[2];
@@ -426,7 +439,7 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
     for (int e = tid; e < RB * RS; e += nthr) reinterpret_cast<float *>(sm4)[e] = 0.f;
     for (int e = tid; e < 2 * (int)(sizeof(WeightTab) / 4); e += nthr) wtab[0].plain[e] = 0.f;
     for (int e = tid; e < 64; e += nthr) s_red[0][e] = 0.f;
-    if (tid < 4) s_alive[tid] = 0;
+    if (tid < kAliveSlots) s_alive[tid] = 0;
     if (tid == 0) s_fail = 0;
     if (__syncthreads_or(bad_geom ? 1 : 0)) {  // nothing issued yet
         if (tid == 0) atomicMax(f.status, ST_ARG);
@@ -553,6 +566,8 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
         mc_next = (float)mcr[i0];
     }
     const bool record = rank == 0 && !replay;
+    // the warp that writes tilts and means: of a cluster the one whose stores nothing waits for
+    const bool recorder = CL ? storer : mover;
     if (record && fresh && tid == 0) {
         thr_[dir == 0 ? 0 : N] = 1.0;
         if (dir == 0) mcr[0] = (double)mean0;
@@ -641,7 +656,7 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
     // The sums' record for the tilt controller, and each row's power of two.
     // False: a row had no usable sum.
     float sc_last = 1.f;            // scales the last summed row
-    int rec_row = -1;               // mover: a row whose mean is to be recorded
+    int rec_row = -1;               // recorder: a row whose mean is to be recorded
     float rec_mean = 0.f;
     __shared__ float s_qs[4];       // storer: scales of the rows to store, the last in entry 3
     int qn = 0, qb = 0;             // how many, buffer of the first
@@ -667,7 +682,7 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
             zexp += e;
             sc_last = inv_pow2(e);
             if (storer && lane == 0) s_qs[3] = sc_last;
-            if (record && dir == 0 && mover && lane == 0) { rec_row = i0 + st; rec_mean = mn; }
+            if (record && dir == 0 && recorder && lane == 0) { rec_row = i0 + st; rec_mean = mn; }
         } else {
             // lane 2 k: sum c of row k; lane 2 k + 1: its first moment
             const float4 ra = *reinterpret_cast<const float4 *>(&s_red[lane & 7][0]);
@@ -685,7 +700,7 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
             const unsigned ok = __ballot_sync(0xffffffffu, c >= 1.2e-38f && co >= 1.2e-38f && co <= 3.0e38f);
             good = (ok & ((0x55u << (2 * k0)) & 0x55u)) == ((0x55u << (2 * k0)) & 0x55u);
             const int row = (lane >> 1) - k0;  // rows since the last time
-            if (record && dir == 0 && mover && lane < 8 && !(lane & 1) && row >= 0) {
+            if (record && dir == 0 && recorder && lane < 8 && !(lane & 1) && row >= 0) {
                 rec_row = i0 + st - (pend - 1 - row);
                 rec_mean = mn;
             }
@@ -778,9 +793,10 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
     // The step's barrier; true where some entry of the new row is not small.
     auto step_sync = [&](int step, bool some) -> bool {
         if constexpr (CL) {
-            if (__any_sync(0xffffffffu, some) && lane < ncta) st_cluster(&s_alive[step & 3], lane, 1);
+            int *const vote = &s_alive[step & (kAliveSlots - 1)];
+            if (__any_sync(0xffffffffu, some) && lane < ncta) st_cluster(vote, lane, 1);
             chain_sync<true>(helper);
-            return s_alive[step & 3] != 0;
+            return *vote != 0;
         } else {
             return __syncthreads_or(some ? 1 : 0) != 0;
         }
@@ -805,6 +821,8 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
     while (st < nsteps) {
         const int steps = steps0 + st;
         const int gave_up = s_fail;
+        // the votes' places of the four steps after this run's (four at most)
+        if (CL && tid < kRunMost) s_alive[(st + kRunMost + tid) & (kAliveSlots - 1)] = 0;
         const bool due = replay || tilt_due(steps);
         const bool summed = pend > 0 && (ready || !alive);
         bool good = true;
@@ -873,9 +891,9 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
             th_tab = tn;
         }
         if (summed || pre) __syncthreads();
-        // FP64 records by the mover, while the others compute
-        if (mover) {
-            if (dir == 0 && tn != theta)
+        // FP64 records, while the other warps compute
+        if (mover || (CL && storer)) {
+            if (mover && dir == 0 && tn != theta)
                 ztilt += (double)(tn - theta) * ((double)n * (i0 + st) + (double)mean);
             if (rec_row >= 0) mcr[rec_row] = (double)rec_mean;
             rec_row = -1;
@@ -896,17 +914,21 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
                 double *tr = thr_ + (dir == 0 ? i0 + st + 1 : i1 - 1 - st);
                 const double tnd = (double)tn;
                 for (;;) {
-                    if (record && lane == 0) *tr = tnd;
+                    if (!CL && record && lane == 0) *tr = tnd;
                     tr += dir == 0 ? 1 : -1;
-                    if (CL && lane == 0) s_alive[(st + u + 2) & 3] = 0;  // read a step ago
                     wait_next();
+                    if (CL) cta_release();
                     alive = step_sync(st + u, false);
                     if (issued < total) issue_next();
                     if (++u == quick || !alive) break;
                 }
             } else if (storer || !has) {  // (a warp without states only keeps the barriers)
                 do {
-                    if (storer) store_row();
+                    if (storer) {
+                        if (CL && record && lane == 0)
+                            thr_[dir == 0 ? i0 + st + u + 1 : i1 - 1 - st - u] = (double)tn;
+                        store_row();
+                    }
                     alive = step_sync(st + u, false);
                 } while (++u < quick && alive);
             } else {
@@ -970,15 +992,16 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
             ready = u + 1 == run && sums;
             bool some = false;
             if (mover) {
-                if (record && lane == 0) thr_[dir == 0 ? i + 1 : i] = (double)tn;
-                if (CL && lane == 0) s_alive[(st + 2) & 3] = 0;  // read a step ago
+                if (!CL && record && lane == 0) thr_[dir == 0 ? i + 1 : i] = (double)tn;
                 for (int k = 0; k + 1 < nck; ++k) {
                     wait_next();
                     __syncthreads();
                     if (issued < total) issue_next();
                 }
                 wait_next();
+                if (CL) cta_release();
             } else if (storer) {
+                if (CL && record && lane == 0) thr_[dir == 0 ? i + 1 : i] = (double)tn;
                 store_row();
                 for (int k = 0; k + 1 < nck; ++k) __syncthreads();
             } else {
@@ -1046,7 +1069,7 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
         failed = !sum_rows(nsteps);
         if (storer)
             while (qn > 0) store_row();
-        if (mover && rec_row >= 0) mcr[rec_row] = (double)rec_mean;
+        if (recorder && rec_row >= 0) mcr[rec_row] = (double)rec_mean;
     }
     if (failed) {
         // Copies already issued must land before the CTA's shared memory is

@@ -449,10 +449,13 @@ void plan_chain(FrameDev &f, int cl, int threads, const ChainAsk &ask) {
     };
     const int need = ask.stages ? ask.stages : 2;
     // four rows are summed together, then stored one a step while the next ones
-    // (and a scaled copy of the last) are written.  A row too long for that is
-    // summed, scaled in place and stored at every step.
+    // (and a scaled copy of the last) are written.  In a cluster two more: another
+    // CTA's next row must not land where this one's storer still reads (its arrival
+    // at a step's barrier orders nothing, see chain_sync).  A row too long for that
+    // is summed, scaled in place and stored at every step.
     f.chainRing = 9;
     if ((size_t)f.chainRing * (f.Mp + 2 * kChainRowPad) * 4 > bud / 2) f.chainRing = 2;
+    else if (cl > 1) f.chainRing = 11;
     // rows are not scaled between sums: a step grows them by at most about
     // 2^{theta n}, theta <= 1.6, which four (two) of them keep within FP32
     f.chainCap = f.chainRing < 4 ? 1 : (f.n <= 15 ? 4 : 2);
