@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(kCrowdMaxThreads, 1) k_chain_crowd(const Frame
     auto issue_next = [&]() {
         const float *src = f.W + (size_t)symbol_of(is_st) * f.wblk + tab.off[is_k];
         uint64_t *b = &bar[is_slot];
-        if (!((f.test_flags & TEST_SKIP_FIRST_COPY) && issued == 0)) {
+        if (!((f.test_flags & TEST_SKIP_COPY) && issued == f.test_copy)) {
             mbar_expect_tx(b, tab.bytes[is_k]);
             bulk_g2s(stage0 + (size_t)is_slot * stageFloats, src, tab.bytes[is_k], b);
         }

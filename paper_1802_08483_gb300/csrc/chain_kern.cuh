@@ -75,6 +75,34 @@ __device__ __forceinline__ void chain_sync(bool relaxed = false) {
 // Orders what this warp saw or wrote before its relaxed arrival, for its own CTA.
 __device__ __forceinline__ void cta_release() { asm volatile("fence.acq_rel.cta;" ::: "memory"); }
 
+// The failure word: one past the step whose barrier the mover of a copy that did not
+// land joins next (kNoFailure: none).  Every warp reads it between two runs of steps
+// and stops if that step lies behind it: a mover that is already in the next run
+// writes a later step, so that all warps of all CTAs stop at the same place,
+// whichever of its writes they saw.
+constexpr int kNoFailure = 0x7fffffff;
+template <bool CL>
+__device__ __forceinline__ int read_failure(const int *word) {
+    int v;
+    if constexpr (CL) asm volatile("ld.relaxed.cluster.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(word)) : "memory");
+    else asm volatile("ld.relaxed.cta.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(word)) : "memory");
+    return v;
+}
+// By the whole warp; the fence orders it before the warp's arrival for every CTA.
+template <bool CL>
+__device__ __forceinline__ void write_failure(int *word, int v, int lane, int ncta) {
+    if constexpr (CL) {
+        if (lane < ncta) {
+            uint32_t a;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(word)), "r"(lane));
+            asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+        }
+        asm volatile("fence.acq_rel.cluster;" ::: "memory");
+    } else if (lane == 0) {
+        asm volatile("st.relaxed.cta.shared::cta.u32 [%0], %1;" ::"r"(smem_u32(word)), "r"(v) : "memory");
+    }
+}
+
 // A lane group: 32 consecutive lanes of one chunk of states, JS = 2^lg adjacent
 // lanes per state (state = s0 + (lane >> lg), below d1).
 struct LaneGroup {
@@ -376,7 +404,7 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
 
     __shared__ uint64_t bar[kMaxStages];
     __shared__ int s_alive[kAliveSlots];  // clusters, by step: some entry >= kRowLow
-    __shared__ int s_fail;      // status of a wait that gave up
+    __shared__ int s_fail;      // see kNoFailure
     __shared__ __align__(16) float s_red[8][8];   // [2 row + (sum, moment)][virtual warp]
     __shared__ __align__(16) WeightTab wtab[2];
     extern __shared__ float4 sm4[];
@@ -440,20 +468,21 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
     for (int e = tid; e < 2 * (int)(sizeof(WeightTab) / 4); e += nthr) wtab[0].plain[e] = 0.f;
     for (int e = tid; e < 64; e += nthr) s_red[0][e] = 0.f;
     if (tid < kAliveSlots) s_alive[tid] = 0;
-    if (tid == 0) s_fail = 0;
+    if (tid == 0) s_fail = kNoFailure;
     if (__syncthreads_or(bad_geom ? 1 : 0)) {  // nothing issued yet
         if (tid == 0) atomicMax(f.status, ST_ARG);
         return;
     }
 
     // The mover's copies: chunk g = (step, k) in order into stage g % NST.
-    const int total = vB > vA ? nsteps * nck : 0;
+    int total = vB > vA ? nsteps * nck : 0;
     int issued = 0, is_k = 0, is_slot = 0;
     const float *is_src = f.W + (size_t)(dir == 0 ? i0 : i1 - 1) * wblk;  // symbol block of the next copy
     const long long is_step = dir == 0 ? wblk : -wblk;
-    const bool skip_first = (f.test_flags & TEST_SKIP_FIRST_COPY) != 0;
+    // testing: a copy that is never issued, every CTA's first or a later one of the last CTA
+    const int skip = (f.test_flags & TEST_SKIP_COPY) && (f.test_copy == 0 || rank == ncta - 1) ? f.test_copy : -1;
     auto issue_next = [&]() {
-        if (lane == 0 && !(skip_first && issued == 0)) {
+        if (lane == 0 && issued != skip) {
             const ChunkGeom g = tab[is_k];
             mbar_expect_tx(&bar[is_slot], g.bytes);
             bulk_g2s(stage0 + (size_t)is_slot * stageFloats, is_src + g.off, g.bytes, &bar[is_slot]);
@@ -462,15 +491,16 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
         if (++is_k == nck) { is_k = 0; is_src += is_step; }
         if (++is_slot == NST) is_slot = 0;
     };
-    // chunk `waited` has landed before the CTA passes the barrier that follows;
-    // a wait that gives up tells every CTA
+    // chunk `waited` has landed before the CTA passes the barrier of `step` that follows;
+    // a wait that gives up tells every CTA, and issues no further copy (its stage's
+    // barrier has not completed the phase that the next copy would count on)
     int waited = 0, wt_slot = 0;
     uint32_t wt_ph = 0;
-    auto wait_next = [&]() {
+    auto wait_next = [&](int step) {
         if (waited >= total) return;
-        if (!mbar_wait(&bar[wt_slot], wt_ph, wait_limit)) {
-            if (CL && lane < ncta) st_cluster(&s_fail, lane, ST_TIMEOUT);
-            if (!CL && lane == 0) s_fail = ST_TIMEOUT;
+        if (!__all_sync(0xffffffffu, mbar_wait(&bar[wt_slot], wt_ph, wait_limit))) {
+            write_failure<CL>(&s_fail, step + 1, lane, ncta);
+            total = issued;
         }
         ++waited;
         if (++wt_slot == NST) { wt_slot = 0; wt_ph ^= 1u; }
@@ -589,7 +619,6 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
     fill_weights(wtab[0], theta);
     if (mover) {
         while (issued < NST && issued < total) issue_next();
-        wait_next();
     }
 
     // Sums of the rows built since the last time (pend of them), in the order of
@@ -816,11 +845,14 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
         q0 = max(0, dir == 0 ? iin0 - i0 : i1 - 1 - iin1);
         q1 = min(nsteps, dir == 0 ? iin1 - i0 + 1 : i1 - iin0);
     }
+    // every CTA of the cluster runs and has set up its shared memory
+    if constexpr (CL) chain_sync<true>();
+    if (mover) wait_next(-1);
     chain_sync<CL>();  // rows, first chunk ready in every CTA
     int st = 0;
     while (st < nsteps) {
         const int steps = steps0 + st;
-        const int gave_up = s_fail;
+        const bool gave_up = read_failure<CL>(&s_fail) <= st;
         // the votes' places of the four steps after this run's (four at most)
         if (CL && tid < kRunMost) s_alive[(st + kRunMost + tid) & (kAliveSlots - 1)] = 0;
         const bool due = replay || tilt_due(steps);
@@ -916,7 +948,7 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
                 for (;;) {
                     if (!CL && record && lane == 0) *tr = tnd;
                     tr += dir == 0 ? 1 : -1;
-                    wait_next();
+                    wait_next(st + u);
                     if (CL) cta_release();
                     alive = step_sync(st + u, false);
                     if (issued < total) issue_next();
@@ -994,11 +1026,11 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
             if (mover) {
                 if (!CL && record && lane == 0) thr_[dir == 0 ? i + 1 : i] = (double)tn;
                 for (int k = 0; k + 1 < nck; ++k) {
-                    wait_next();
+                    wait_next(st);
                     __syncthreads();
                     if (issued < total) issue_next();
                 }
-                wait_next();
+                wait_next(st);
                 if (CL) cta_release();
             } else if (storer) {
                 if (CL && record && lane == 0) thr_[dir == 0 ? i + 1 : i] = (double)tn;
@@ -1058,7 +1090,8 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
             cur = nxt;
         }
     }
-    if (!failed && s_fail) failed = true;
+    const bool gave_up = read_failure<CL>(&s_fail) <= st;
+    if (gave_up) failed = true;
     if (!failed && pend > 0) {  // the last rows (the last step's sums are ready)
         if (storer)
             while (qn > 0) store_row();
@@ -1077,7 +1110,7 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
         if (mover)
             for (int h = max(0, issued - NST); h < issued; ++h)
                 mbar_wait(&bar[h % NST], (uint32_t)((h / NST) & 1), wait_limit);
-        if (tid == 0) atomicMax(f.status, s_fail ? s_fail : ST_ZERO);
+        if (tid == 0) atomicMax(f.status, gave_up ? ST_TIMEOUT : ST_ZERO);
         __syncthreads();
         return;
     }

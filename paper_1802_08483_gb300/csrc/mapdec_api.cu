@@ -317,10 +317,11 @@ void plan_shape(FrameDev &f, const mapdec_frame_desc_t &d, bool grad, int forceP
     f.chain_flags = 0;
     // bounded waits: a recursion gives up on a copy after this many polls
     f.wait_limit = 1u << 26;
-    f.test_flags = 0;
+    f.test_flags = f.test_copy = 0;
     if (const char *e = std::getenv("MAPDEC_TEST_STALL_CHAIN")) {  // testing: the timeout path
-        if (std::atoi(e) == 1) {
-            f.test_flags |= TEST_SKIP_FIRST_COPY;
+        if (std::atoi(e) >= 1) {
+            f.test_flags |= TEST_SKIP_COPY;
+            f.test_copy = std::atoi(e) - 1;
             f.wait_limit = 4096;
         }
     }

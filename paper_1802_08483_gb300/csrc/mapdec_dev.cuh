@@ -18,7 +18,7 @@ constexpr int CH_SEGMENTED = 1;   // start/end rows and controller state come fr
 constexpr int CH_REPLAY = 2;      // forward chain replays the recorded tilts (recompute sweep)
 
 // test_flags
-constexpr int TEST_SKIP_FIRST_COPY = 1;  // a recursion's first copy is never issued
+constexpr int TEST_SKIP_COPY = 1;  // one of a recursion's copies is never issued
 
 constexpr int kMaxI = 7;        // insertion cap supported by the kernels
 constexpr int kMaxMN = 64;      // n(I+1) + 1 <= 64 (received window fits 64 bits)
@@ -83,7 +83,8 @@ struct FrameDev {
     int chainVWarps;  // virtual warps with lanes (<= 8)
     int chainWarps, chainList;  // compute warps of the launch, lane groups of one (and an end mark)
     uint32_t wait_limit;  // polls before a recursion's wait on a copy gives up (ST_TIMEOUT)
-    int test_flags;       // TEST_SKIP_FIRST_COPY: the first copy is never issued (tests the timeout path)
+    int test_flags;       // TEST_SKIP_COPY: copy number test_copy is never issued (tests the timeout path)
+    int test_copy;
     long long rho;
     long long wblk;  // floats per symbol block of W (M * MNS rounded up to 4)
     // FP32 lattice constants.  Every received bit carries a weight kappa: the
