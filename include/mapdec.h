@@ -202,8 +202,9 @@ typedef struct {
  * Results equal mapdec_decode's.  All scratch lives in one static device
  * array of 32 MiB per GPU that loads the library, held until the process
  * exits; a frame whose scratch does not fit is rejected with
- * MAPDEC_ERR_TOO_LARGE (about N * (2 xmax + 1) * (n(I+1)+1) * 4 bytes for the
- * transition sums dominates).  The first call on a device looks up the
+ * MAPDEC_ERR_TOO_LARGE.  The transition sums take about N * (2 xmax + 1) *
+ * (n(I+1)+1) * 4 bytes; next come the APP partial sums, for which frames near the
+ * limit take longer tiles (and more time) than mapdec_decode.  The first call on a device looks up the
  * array's address on that device; make that first call before any stream
  * capture.  Every call shares the array and leaves its contents behind (the
  * next call clears what must start at zero), so calls whose work overlaps on

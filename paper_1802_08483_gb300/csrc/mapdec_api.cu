@@ -1601,7 +1601,9 @@ void load_inputs(mapdec_batch *b, const uint8_t *rx_all, const float *priors_all
 // whole scratch of one decode (descriptor, work lists, packed bits, W, alpha,
 // beta, APP partial sums, status) is carved out of the file-scope array
 // below, which every GPU that loads the library holds until the process
-// exits.  Nothing is allocated per call, on the device or on the host.
+// exits.  Nothing is allocated per call, on the device or on the host.  The
+// descriptor has its place behind the arena, so that its size does not move the
+// line between frames that fit and frames that do not.
 // ---------------------------------------------------------------------------
 namespace {
 
@@ -1618,7 +1620,7 @@ void *g_static_addr[kStaticMaxDevices] = {};
 
 }  // namespace
 
-static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
+static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes + sizeof(FrameDev)];
 
 namespace {
 
@@ -1670,6 +1672,66 @@ __global__ void k_static_setup(FrameDev f, FrameDev *fdst, Work *fwd, int T, Wor
         rxwp[0] = rxw;
         *status = 0;
     }
+}
+
+// Places of one decode's regions in the arena (each 256-byte aligned).
+struct StaticLayout {
+    size_t fwd, bwd, chain, fin, rxp, rxwp, rxw, cw, pri, W, a, b, Lp, thf, mcf, thb, st, total;
+};
+long long static_rx_words(const mapdec_frame_desc_t &d) { return (d.rx_len + 31) / 32 + 4; }
+StaticLayout static_layout(const FrameDev &f, const mapdec_frame_desc_t &d, bool priors) {
+    StaticLayout L;
+    size_t off = 0;
+    auto take = [&](size_t bytes) -> size_t {
+        const size_t o = off;
+        off += rup(bytes, 256);
+        return o;
+    };
+    L.fwd = take(sizeof(Work) * (size_t)f.Tf);
+    L.bwd = take(sizeof(Work) * (size_t)f.T2);
+    L.chain = take(sizeof(Work) * 2);
+    L.fin = take(sizeof(Work) * (size_t)finalize_chunks(d.N));
+    L.rxp = take(sizeof(void *));
+    L.rxwp = take(sizeof(void *));
+    L.rxw = take(4 * (size_t)static_rx_words(d));
+    L.cw = take(4 * (size_t)d.q);
+    L.pri = priors ? off : take(4 * (size_t)d.N * d.q);
+    L.W = take(4 * ((size_t)f.N * f.wblk + 16));
+    L.a = take(4 * (size_t)(f.N + 1) * f.Mp);
+    L.b = take(4 * (size_t)(f.N + 1) * f.Mp);
+    L.Lp = take(4 * (size_t)f.T2 * f.S2 * f.q);
+    L.thf = take(8 * (size_t)(f.N + 1));
+    L.mcf = take(8 * (size_t)(f.N + 1));
+    L.thb = take(8 * (size_t)(f.N + 1));
+    L.st = take(sizeof(int));
+    L.total = off;
+    return L;
+}
+
+// Tiles of an allocation-free decode: those of mapdec_decode where their scratch
+// fits the arena.  Short tiles multiply the rows of APP partial sums (q = 64, n = 8,
+// N = 660, xmax = 220: 31.1 MiB of scratch as plan_shape has them, 36.6 with short
+// ones), so a larger frame takes the shortest super-tiles that fit, and plan_shape's
+// tiles at the end.  False: not even those fit.
+bool plan_static(FrameDev &f, const mapdec_frame_desc_t &d, bool priors, StaticLayout &L) {
+    const FrameDev planned = f;
+    const long long pos = (long long)f.n * f.N + f.xmax + 1;
+    const int most = supertile_split(most_supertiles(f));
+    split_supertiles(f, most);
+    fit_app_tile(f, pos);
+    fit_fwd_tile(f, pos, false);
+    L = static_layout(f, d, priors);
+    for (int k = most; k >= 1 && L.total > kStaticScratchBytes; k /= 2) {
+        f = planned;
+        split_supertiles(f, k);
+        fit_fwd_tile(f, pos, false);
+        L = static_layout(f, d, priors);
+    }
+    if (L.total > kStaticScratchBytes) {
+        f = planned;
+        L = static_layout(f, d, priors);
+    }
+    return L.total <= kStaticScratchBytes;
 }
 
 bool device_pointer(const void *p) {
@@ -2159,54 +2221,25 @@ int mapdec_decode_noalloc(const mapdec_frame_desc_t *frame, const uint8_t *rx_de
 
     FrameDev f{};
     plan_shape(f, d, false, 0);
-    const long long pos = (long long)f.n * f.N + f.xmax + 1;
-    split_supertiles(f, supertile_split(most_supertiles(f)));
-    fit_app_tile(f, pos);
-    fit_fwd_tile(f, pos, false);
+    StaticLayout L;
+    if (!plan_static(f, d, priors_dev != nullptr, L)) return MAPDEC_ERR_TOO_LARGE;
     const int cl = chain_cluster(2, f.chainNV);
     const int cthr = chain_threads(cl, f.chainVWarps, f.chainNV);
     plan_chain(f, cl, cthr, chain_ask(nullptr));
     const bool crowd = crowd_launch(2) || chain_smem_bytes(f) > kChainSmemMost;
-    // carve the arena (every region 256-byte aligned)
-    size_t off = 0;
-    auto take = [&](size_t bytes) -> size_t {
-        const size_t o = off;
-        off += rup(bytes, 256);
-        return o;
-    };
-    const size_t o_frame = take(sizeof(FrameDev));
-    const size_t o_fwd = take(sizeof(Work) * (size_t)f.Tf);
-    const size_t o_bwd = take(sizeof(Work) * (size_t)f.T2);
-    const size_t o_chain = take(sizeof(Work) * 2);
     const int nfin = finalize_chunks(d.N);
-    const size_t o_fin = take(sizeof(Work) * (size_t)nfin);
-    const size_t o_rxp = take(sizeof(void *));
-    const size_t o_rxwp = take(sizeof(void *));
-    const long long nwords = (d.rx_len + 31) / 32 + 4;
-    const size_t o_rxw = take(4 * (size_t)nwords);
-    const size_t o_cw = take(4 * (size_t)d.q);
-    const size_t o_pri = priors_dev ? off : take(4 * (size_t)d.N * d.q);
-    const size_t o_W = take(4 * ((size_t)f.N * f.wblk + 16));
-    const size_t o_a = take(4 * (size_t)(f.N + 1) * f.Mp);
-    const size_t o_b = take(4 * (size_t)(f.N + 1) * f.Mp);
-    const size_t o_Lp = take(4 * (size_t)f.T2 * f.S2 * f.q);
-    const size_t o_thf = take(8 * (size_t)(f.N + 1));
-    const size_t o_mcf = take(8 * (size_t)(f.N + 1));
-    const size_t o_thb = take(8 * (size_t)(f.N + 1));
-    const size_t o_st = take(sizeof(int));
-    if (off > kStaticScratchBytes) return MAPDEC_ERR_TOO_LARGE;
 
     unsigned char *A = (unsigned char *)base;
-    f.rxbits = (const uint32_t *)(A + o_rxw);
-    f.cw = (const uint32_t *)(A + o_cw);
-    f.priors = priors_dev ? priors_dev : (const float *)(A + o_pri);
-    f.W = (float *)(A + o_W);
-    f.alpha = (float *)(A + o_a);
-    f.beta = (float *)(A + o_b);
-    f.Lp = (float *)(A + o_Lp);
-    f.thf = (double *)(A + o_thf);
-    f.mcf = (double *)(A + o_mcf);
-    f.thb = (double *)(A + o_thb);
+    f.rxbits = (const uint32_t *)(A + L.rxw);
+    f.cw = (const uint32_t *)(A + L.cw);
+    f.priors = priors_dev ? priors_dev : (const float *)(A + L.pri);
+    f.W = (float *)(A + L.W);
+    f.alpha = (float *)(A + L.a);
+    f.beta = (float *)(A + L.b);
+    f.Lp = (float *)(A + L.Lp);
+    f.thf = (double *)(A + L.thf);
+    f.mcf = (double *)(A + L.mcf);
+    f.thb = (double *)(A + L.thb);
     f.Gp = nullptr;
     f.Gc = nullptr;
     f.Rout = nullptr;
@@ -2214,21 +2247,22 @@ int mapdec_decode_noalloc(const mapdec_frame_desc_t *frame, const uint8_t *rx_de
     f.dpriors = nullptr;
     f.loglik = loglik_dev;
     f.dchan = nullptr;
-    f.status = (int *)(A + o_st);
+    f.status = (int *)(A + L.st);
 
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    FrameDev *fdev = (FrameDev *)(A + o_frame);
-    Work *wf = (Work *)(A + o_fwd), *wb = (Work *)(A + o_bwd), *wc = (Work *)(A + o_chain);
-    Work *wfin = (Work *)(A + o_fin);
+    FrameDev *fdev = (FrameDev *)(A + kStaticScratchBytes);
+    Work *wf = (Work *)(A + L.fwd), *wb = (Work *)(A + L.bwd), *wc = (Work *)(A + L.chain);
+    Work *wfin = (Work *)(A + L.fin);
+    const long long nwords = static_rx_words(d);
     const long long nuni = priors_dev ? 0 : (long long)d.N * d.q;
     k_static_setup<<<64, 256, 0, s>>>(f, fdev, wf, f.Tf, wb, f.T2, wc, wfin, nfin,
-                                      (const uint8_t **)(A + o_rxp), (uint32_t **)(A + o_rxwp),
-                                      rx_dev, (uint32_t *)(A + o_rxw), (uint32_t *)(A + o_cw), cb,
-                                      d.q, (float *)(A + o_pri), nuni, 1.0f / (float)d.q,
+                                      (const uint8_t **)(A + L.rxp), (uint32_t **)(A + L.rxwp),
+                                      rx_dev, (uint32_t *)(A + L.rxw), (uint32_t *)(A + L.cw), cb,
+                                      d.q, (float *)(A + L.pri), nuni, 1.0f / (float)d.q,
                                       f.status);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess)
-        e = launch_pack(fdev, (const uint8_t *const *)(A + o_rxp), (uint32_t *const *)(A + o_rxwp), 1,
+        e = launch_pack(fdev, (const uint8_t *const *)(A + L.rxp), (uint32_t *const *)(A + L.rxwp), 1,
                         nwords, s);
     if (e == cudaSuccess) e = launch_fwd(d.n, d.I, fdev, wf, f.Tf, fwd_smem_bytes(f), s);
     if (e == cudaSuccess)
