@@ -215,6 +215,7 @@ struct FrameHost {
     bool tcb = false;       // APP producer on the tensor cores
     bool split = false;     // APP super-tiles may be shortened to fill the GPU
     bool fit = false;       // and tiles
+    bool rows = false;      // APP partial sums may be kept per sub-tile (gradients)
     std::vector<float> phi0, phiN;  // boundary drift priors (stream decoding), or empty
     int64_t phi_off = 0;    // float offset of phi0 (then phiN) in the batch's buffer
 };
@@ -652,6 +653,29 @@ void split_supertiles(FrameDev &f, int d) {
     f.T2 = (f.T + f.nsub - 1) / f.nsub;
 }
 
+// The tiles of a planned frame in a launch of `pos` received positions and `ctas` APP
+// CTAs (gradients: sub-tiles) in all.  fill: short enough for the launch to fill the
+// GPU; else the planner's APP tiles.
+void fill_tiles(FrameHost &h, long long pos, long long ctas, bool grad, bool fill) {
+    FrameDev &f = h.dev;
+    if (fill && h.fit && h.split) fit_app_tile(f, pos);
+    if (h.fit && !h.tc && (fill || !h.store)) fit_fwd_tile(f, pos, grad);
+    if (fill && h.split) split_supertiles(f, supertile_split(ctas));
+    if (fill && h.rows) {
+        // eight CTAs per SM, no more sub-tiles each than planned; the order of the sums
+        // stays that of the planned super-tiles.  A launch that has as many CTAs with
+        // those keeps their rows: rows per sub-tile are up to twice a frame's scratch.
+        const int sms = device_sms() > 0 ? device_sms() : 152;
+        const int nsub = (int)std::max(1LL, std::min<long long>(f.nsub, ctas / (8LL * sms)));
+        if (nsub == 1 || nsub < f.nsub) {
+            f.group = f.nsub;
+            f.S2 = f.S;
+            f.nsub = nsub;
+            f.T2 = (f.T + nsub - 1) / nsub;
+        }
+    }
+}
+
 double frame_cost(const FrameDev &f) {
     // algorithmic flop estimate used for load balancing and reporting
     const double cells = (f.I + 1) * f.n * (f.n + 1) / 2.0 + (f.n + 1);
@@ -1031,12 +1055,11 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
                                                   : (long long)h.d.n * h.d.N + h.d.xmax + 1;
         // stored metrics: both producers on one tile, so only where both are fitted
         h.fit = !per_sym && (!h.store || h.split) && !(tuned && tu.P > 0) && (plain || forceP <= 0);
-        if (b->grad && !per_sym) {
-            // partial sums per sub-tile; the order of the sums stays that of the
-            // planned super-tiles
-            h.dev.group = h.dev.nsub;
-            h.dev.S2 = h.dev.S;
-            class_ctas[{h.d.n, h.d.I}] += b->segmented ? seg_row_tiles(h.dev, h.segK) - 2 : h.dev.T;
+        h.rows = b->grad && !per_sym;
+        if (h.rows) {
+            FrameDev t = h.dev;
+            t.group = t.nsub;
+            class_ctas[{h.d.n, h.d.I}] += b->segmented ? seg_row_tiles(t, h.segK) - 2 : h.dev.T;
         }
         if (h.split)
             class_ctas[{h.d.n, h.d.I}] += b->segmented ? seg_row_tiles(h.dev, h.segK) - 2
@@ -1052,24 +1075,6 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
         b->cw_total += (int64_t)h.cw.size();
         h.phi_off = b->phi_total;
         b->phi_total += (int64_t)(h.phi0.size() + h.phiN.size());
-    }
-    for (auto &h : b->fr) {
-        const long long pos = class_pos[{h.d.n, h.d.I}];
-        if (h.fit && h.split) fit_app_tile(h.dev, pos);
-        if (h.fit && !h.tc) fit_fwd_tile(h.dev, pos, b->grad);
-        if (h.split) split_supertiles(h.dev, supertile_split(class_ctas[{h.d.n, h.d.I}]));
-        if (h.dev.group) {  // eight CTAs per SM, no more sub-tiles each than planned
-            const int sms = device_sms() > 0 ? device_sms() : 152;
-            h.dev.nsub = (int)std::max(1LL, std::min<long long>(
-                h.dev.group, class_ctas[{h.d.n, h.d.I}] / (8LL * sms)));
-            h.dev.T2 = (h.dev.T + h.dev.nsub - 1) / h.dev.nsub;
-        }
-        if (b->segmented) {
-            h.scratch_floats = frame_scratch_floats_seg(h.dev, h.segK, h.nseg, b->grad);
-        } else {
-            h.scratch_floats = frame_scratch_floats(h.dev, b->grad);
-            if (h.store) h.scratch_floats += rup(metric_store_floats(h.dev), 64);
-        }
     }
     // resident buffers
     b->d_rx = (uint8_t *)b->dalloc(b->rx_total + 64);
@@ -1105,11 +1110,54 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
     size_t freeb = 0, totb = 0;
     CK(cudaMemGetInfo(&freeb, &totb));
     size_t bud = budget > 0 ? (size_t)budget : (size_t)(0.6 * (double)freeb);
-    size_t maxf = 0, sumf = 0;
-    for (auto &h : b->fr) { maxf = std::max(maxf, h.scratch_floats); sumf += h.scratch_floats; }
-    const bool one_wave = sumf * 4 <= bud;
-    size_t wave_bud = one_wave ? bud / 4 : bud / 4 / kRegions;  // in floats
-    if (wave_bud < maxf) wave_bud = maxf;                        // at least one frame per wave
+    // Short tiles and partial sums per sub-tile cost scratch (gradients with q = 64,
+    // n = 12, I = 2, xmax = 100: 60 KB a symbol against 32).  The planner's tiles stay
+    // where the batch then fits its budget in one wave or in fewer: several waves run
+    // the slower recursions, and more than the tiles gain is lost.
+    std::vector<FrameDev> planned(nf);
+    for (int i = 0; i < nf; ++i) planned[i] = b->fr[i].dev;
+    struct Need {
+        size_t wave_bud = 0;  // in floats
+        bool one_wave = false;
+        int waves = 0;
+    };
+    auto plan_tiles = [&](bool fill) {
+        size_t maxf = 0, sumf = 0;
+        for (int i = 0; i < nf; ++i) {
+            FrameHost &h = b->fr[i];
+            h.dev = planned[i];
+            const std::pair<int, int> cls{h.d.n, h.d.I};
+            fill_tiles(h, class_pos[cls], class_ctas[cls], b->grad, fill);
+            if (b->segmented) {
+                h.scratch_floats = frame_scratch_floats_seg(h.dev, h.segK, h.nseg, b->grad);
+            } else {
+                h.scratch_floats = frame_scratch_floats(h.dev, b->grad);
+                if (h.store) h.scratch_floats += rup(metric_store_floats(h.dev), 64);
+            }
+            maxf = std::max(maxf, h.scratch_floats);
+            sumf += h.scratch_floats;
+        }
+        Need w;
+        w.one_wave = sumf * 4 <= bud;
+        w.wave_bud = w.one_wave ? bud / 4 : bud / 4 / kRegions;
+        if (w.wave_bud < maxf) w.wave_bud = maxf;  // at least one frame per wave
+        size_t acc = 0;
+        for (auto &h : b->fr) {
+            if (w.waves == 0 || acc + h.scratch_floats > w.wave_bud) {
+                ++w.waves;
+                acc = 0;
+            }
+            acc += h.scratch_floats;
+        }
+        return w;
+    };
+    Need need = plan_tiles(true);
+    if (!need.one_wave) {
+        const Need own = plan_tiles(false);
+        if (own.one_wave || own.waves < need.waves) need = own;
+        else need = plan_tiles(true);
+    }
+    const size_t wave_bud = need.wave_bud;
     {
         size_t acc = 0;
         Wave w;

@@ -68,8 +68,8 @@ struct FrameDev {
     const float *phi0, *phiN;
     int nsub;     // sub-tiles per backward super-tile (the work of one CTA)
     int T2;       // backward super-tiles: ceil(T / nsub)
-    int group;    // gradient mode: the APP producer keeps the partial sums of every
-                  // sub-tile, and finalize adds them up group sub-tiles at a time;
+    int group;    // > 0 (gradient frames): the APP producer keeps the partial sums of
+                  // every sub-tile, and finalize adds them up group sub-tiles at a time;
                   // 0: the partial sums of a super-tile
     int S2;       // rows of Lp per sub-tile (group > 0) or super-tile: the symbols it touches
     // Recursions (k_chain).  Summation order: chunks of chainCD states, chainVW
@@ -107,7 +107,7 @@ struct FrameDev {
     float *alpha;    // (N+1) * Mp normalised forward rows
     float *beta;     // (N+1) * Mp normalised backward rows
     float *Lp;       // S2 * q  partial unnormalised APP sums per sub- or super-tile
-    float *Gp;       // S2 * 3  partial tangent sums per sub-tile (gradient mode)
+    float *Gp;       // S2 * 3  partial tangent sums per sub- or super-tile (gradient mode)
     float *Rout;     // receiver-metric dump (debug entry), (rho+1)*q*MN or null
     float *Rg;       // stored receiver metrics (or null: recompute), T * P*MN * DS:
                      // tile t at t*P*MN*DS, row pl*MN + j, column D (DS = roundup4(q))

@@ -307,11 +307,12 @@ __device__ __forceinline__ void window_tilt(int S, int S4, int P, int BW, float 
 // ---------------------------------------------------------------------------
 // Backward producer (APP partial sums, optional tangents).  One CTA owns a
 // super-tile of nsub sub-tiles of P positions and accumulates, in shared
-// memory, for every symbol i it touches (frames planned for gradients, f.group > 0,
-// in decode calls too: stores for every sub-tile, so that the CTAs can be short
-// enough to fill the GPU while finalize adds the sub-tiles up in one fixed order;
-// 48 frames N = 2000, q = 32, segments of 45 symbols: super-tiles of 42 sub-tiles
-// were 144 CTAs a launch, the whole pass 67.4 ms; of 3 sub-tiles 41.3 ms):
+// memory, for every symbol i it touches (gradient frames of launches that planned
+// super-tiles cannot fill, f.group > 0, in decode calls too: stores for every
+// sub-tile, so that the CTAs can be short enough to fill the GPU while finalize adds
+// the sub-tiles up in one fixed order; 48 frames N = 2000, q = 32, segments of 45
+// symbols: super-tiles of 42 sub-tiles were 144 CTAs a launch, the whole pass
+// 67.4 ms; of 3 sub-tiles 41.3 ms):
 //   Lacc[i][D] = sum_{p in super-tile, j} alpha_i(s') R[p][D][j] beta_{i+1}(s'+j-n)
 //   Gacc[i][t] = sum_D prior_i(D) (the same sum with the t-th tangent of R)
 // Per sub-tile the contraction is evaluated as
@@ -320,7 +321,8 @@ __device__ __forceinline__ void window_tilt(int S, int S4, int P, int BW, float 
 // A operand AB = alpha (x) beta factored, so it is never materialised.
 // smem: Rt[K][CW]  (K = P*MN, CW = NR*DS, DS = roundup4(q); column t*DS + D)
 //       Aw[P][S4], Bw[BW][S4] (BW = P + MN - 1), both carrying the tilt factors
-//       symbol constants (4 x S4), Lacc[S2][q] or (gradient) Ct[3][S4][DS]
+//       symbol constants (4 x S4), Lacc[S2][q] and Gacc[S2][3] (group = 0),
+//       Ct[3][S4][DS] (gradient)
 // ---------------------------------------------------------------------------
 template <int NB, int IB, bool GRAD>
 __global__ void __launch_bounds__(kThreads, (GRAD && (NB == 0 || NB > 10)) ? 1 : 2) k_bwd(const FrameDev *__restrict__ frames,
@@ -351,11 +353,15 @@ __global__ void __launch_bounds__(kThreads, (GRAD && (NB == 0 || NB > 10)) ? 1 :
     float *symG = symF + Smax4;                                 // its slope in pl
     float *symPhi = symG + Smax4;                               // theta'_{i+1} - 1
     float *Lacc = symPhi + Smax4;
-    float *Ct = Lacc;  // gradient mode (no accumulators)
-    const bool apart = GRAD || f.group != 0;  // rows of Lp per sub-tile
+    const bool apart = f.group != 0;  // rows of Lp and Gp per sub-tile, no accumulators
+    float *Gacc = Lacc + (((size_t)f.S2 * q + 3) & ~(size_t)3);
+    float *Ct = apart ? Lacc : Gacc + (((size_t)f.S2 * 3 + 3) & ~(size_t)3);
 
-    if (!apart)
+    if (!apart) {
         for (int idx = threadIdx.x; idx < S2 * q; idx += blockDim.x) Lacc[idx] = 0.f;
+        if (GRAD)
+            for (int idx = threadIdx.x; idx < S2 * 3; idx += blockDim.x) Gacc[idx] = 0.f;
+    }
 
     for (int sub = 0; sub < f.nsub; ++sub) {
         const long long p0 = ((long long)wk.tile * f.nsub + sub) * P;
@@ -502,7 +508,8 @@ __global__ void __launch_bounds__(kThreads, (GRAD && (NB == 0 || NB > 10)) ? 1 :
                 const float *ct = Ct + ((size_t)tt * Smax4 + il) * DS;
                 float s = 0.f;
                 for (int D = 0; D < q; ++D) s = fmaf(__ldg(pr + D), ct[D], s);
-                f.Gp[(row0 + il) * 3 + tt] = s;
+                if (apart) f.Gp[(row0 + il) * 3 + tt] = s;
+                else Gacc[(off + il) * 3 + tt] += s;
             }
         }
         __syncthreads();
@@ -511,6 +518,9 @@ __global__ void __launch_bounds__(kThreads, (GRAD && (NB == 0 || NB > 10)) ? 1 :
     const size_t row0 = (size_t)wk.tile * f.S2;
     for (int idx = threadIdx.x; idx < S2 * q; idx += blockDim.x)
         f.Lp[row0 * q + idx] = Lacc[idx];
+    if (GRAD)
+        for (int idx = threadIdx.x; idx < S2 * 3; idx += blockDim.x)
+            f.Gp[row0 * 3 + idx] = Gacc[idx];
 }
 
 // Step (1) alone: one thread per (p, D).

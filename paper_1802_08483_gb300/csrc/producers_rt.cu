@@ -31,9 +31,9 @@ size_t bwd_smem_bytes(const FrameDev &f, bool grad) {
     const size_t BW = (size_t)f.P + f.MN - 1;
     size_t fl = K * NR * DS + (size_t)f.P * Smax4 + BW * Smax4 + 4 * Smax4;
     if (grad) fl += 3 * Smax4 * DS;
-    // the accumulators: none in gradient mode, but tiles are planned with room for
-    // them (the tiles fix the order of the gradient's sums)
-    if (!grad || f.group == 0)
+    // the accumulators: none with rows per sub-tile, but tiles are planned with room
+    // for them (the tiles fix the order of the gradient's sums)
+    if (f.group == 0)
         fl += (((size_t)f.S2 * f.q + 3) & ~(size_t)3) + (((size_t)f.S2 * 3 + 3) & ~(size_t)3);
     return 4 * fl;
 }
