@@ -4,8 +4,7 @@
 
 #include <type_traits>
 
-#include "mapdec_dev.cuh"
-#include "mapdec_kernels.h"
+#include "chain_crowd.cuh"
 
 namespace mdk {
 
@@ -16,17 +15,16 @@ constexpr int kChainMostThreads = 320;  // one CTA: 8 virtual warps, mover and s
 // the partial sums), a CTA with a warp per lane group (rows of several chunks; the
 // partial sums are read back from the rows), a cluster of such CTAs.
 constexpr int kChainNarrow = 0, kChainWide = 1, kChainCluster = 2;
-constexpr int kMaxStages = 8;
 
-// Tilt controller (see k_chain).
-constexpr float kTiltGainMin = 0.02f;  // long-run smoothing of the entropy-rate estimate
-constexpr float kTiltStepMax = 0.02f;  // largest change of the tilt between two rows
-constexpr float kTiltMin = 0.2f, kTiltMax = 1.6f;
-constexpr int kTiltEvery = 4;    // steps between tilt updates once settled
-constexpr int kTiltSettle = 64;  // updates every step for the first steps
 // Rows are divided by their power of two when their sums are formed (at tilt
 // updates), or at once when their largest entry fell below this.
 constexpr float kRowLow = 1.f / 65536.f;
+// A sum of rows that were not scaled one by one is not used below this (2^-64): a step
+// may have cost entries that a row scaled at once would have kept.  The launch is then
+// run again with every row scaled (crowd_again), as where a sum left FP32's range:
+// priors are used as given, whatever their rows' sums, and four steps may multiply a
+// row by what a step may (2^+-126).
+constexpr float kSumLow = 1.f / 18446744073709551616.f;
 constexpr int kRunMost = 4;      // rows between two sums, at most
 constexpr int kAliveSlots = 16;  // steps until a vote's place is used again (a power of two)
 
@@ -726,7 +724,7 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
             const float co = c * inv_pow2(dp);
             const float lc = log2f(co);
             mn = cm / c;
-            const unsigned ok = __ballot_sync(0xffffffffu, c >= 1.2e-38f && co >= 1.2e-38f && co <= 3.0e38f);
+            const unsigned ok = __ballot_sync(0xffffffffu, c >= kSumLow && c <= 3.0e38f && co >= 1.2e-38f && co <= 3.0e38f);
             good = (ok & ((0x55u << (2 * k0)) & 0x55u)) == ((0x55u << (2 * k0)) & 0x55u);
             const int row = (lane >> 1) - k0;  // rows since the last time
             if (record && dir == 0 && recorder && lane < 8 && !(lane & 1) && row >= 0) {
@@ -1106,12 +1104,16 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
     }
     if (failed) {
         // Copies already issued must land before the CTA's shared memory is
-        // released: wait for them, again with a bound.
+        // released or used again: wait for them, again with a bound.
+        bool late = gave_up;
         if (mover)
             for (int h = max(0, issued - NST); h < issued; ++h)
-                mbar_wait(&bar[h % NST], (uint32_t)((h / NST) & 1), wait_limit);
-        if (tid == 0) atomicMax(f.status, gave_up ? ST_TIMEOUT : ST_ZERO);
-        __syncthreads();
+                late |= !mbar_wait(&bar[h % NST], (uint32_t)((h / NST) & 1), wait_limit);
+        late = __syncthreads_or(late ? 1 : 0) != 0;
+        if (late && tid == 0) atomicMax(f.status, ST_TIMEOUT);
+        if (gave_up) return;  // the same in every CTA
+        if constexpr (CL) chain_sync<true>();  // the other CTAs' parts of rows that are stored again
+        if (rank == 0 && !late) crowd_again(&f, dir | (replay ? 2 : 0));
         return;
     }
     const float *last = rows + cur;

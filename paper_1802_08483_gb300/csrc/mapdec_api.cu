@@ -459,7 +459,8 @@ void plan_chain(FrameDev &f, int cl, int threads, const ChainAsk &ask) {
     if ((size_t)f.chainRing * (f.Mp + 2 * kChainRowPad) * 4 > bud / 2) f.chainRing = 2;
     else if (cl > 1) f.chainRing = 11;
     // rows are not scaled between sums: a step grows them by at most about
-    // 2^{theta n}, theta <= 1.6, which four (two) of them keep within FP32
+    // 2^{theta n}, theta <= 1.6, which four (two) of them keep within FP32 where the
+    // priors' rows sum to about 1 (for others see kSumLow)
     f.chainCap = f.chainRing < 4 ? 1 : (f.n <= 15 ? 4 : 2);
     int ck = f.chainVC;
     for (int nck = 1; nck <= f.chainVC; ++nck) {
@@ -477,6 +478,12 @@ void plan_chain(FrameDev &f, int cl, int threads, const ChainAsk &ask) {
     if (!ask.stages)
         while (stages < 8 && fits(ck, stages + 1, bud)) ++stages;
     fits(ck, stages, bud);
+}
+
+// Shared memory of a k_chain launch: room for k_chain_crowd's rows and stages too, which
+// it falls back on (crowd_again).
+size_t chain_launch_smem(const FrameDev &f) {
+    return std::max(chain_smem_bytes(f), crowd_smem_bytes(f));
 }
 
 // Block size of a recursion launch over frames with at most maxVW virtual warps
@@ -1204,7 +1211,7 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
         for (int i = w.f0; i < w.f1; ++i) {
             FrameHost &h = b->fr[i];
             plan_chain(h.dev, w.chain_cl, w.chain_thr, h.chain);
-            if (chain_smem_bytes(h.dev) > kChainSmemMost) w.crowd = true;  // rows too long for k_chain
+            if (chain_launch_smem(h.dev) > kChainSmemMost) w.crowd = true;  // rows too long for k_chain
             FrameDev f = h.dev;
             f.rxbits = b->d_rxw + h.rxw_off;
             f.cw = b->d_cw + h.cw_off;
@@ -1302,7 +1309,7 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
                 const int mn = apart ? devs[k].MN : w.chain_mn;
                 per[mn].push_back({k, 0});
                 per[mn].push_back({k, 1});
-                csm[mn] = std::max(csm[mn], w.crowd ? crowd_smem_bytes(devs[k]) : chain_smem_bytes(devs[k]));
+                csm[mn] = std::max(csm[mn], w.crowd ? crowd_smem_bytes(devs[k]) : chain_launch_smem(devs[k]));
                 w.smem_chain = std::max(w.smem_chain, csm[mn]);
             }
             for (auto &kv : per) {
@@ -2274,7 +2281,7 @@ int mapdec_decode_noalloc(const mapdec_frame_desc_t *frame, const uint8_t *rx_de
     const int cl = chain_cluster(2, f.chainNV);
     const int cthr = chain_threads(cl, f.chainVWarps, f.chainNV);
     plan_chain(f, cl, cthr, chain_ask(nullptr));
-    const bool crowd = crowd_launch(2) || chain_smem_bytes(f) > kChainSmemMost;
+    const bool crowd = crowd_launch(2) || chain_launch_smem(f) > kChainSmemMost;
     const int nfin = finalize_chunks(d.N);
 
     unsigned char *A = (unsigned char *)base;
@@ -2315,7 +2322,7 @@ int mapdec_decode_noalloc(const mapdec_frame_desc_t *frame, const uint8_t *rx_de
     if (e == cudaSuccess) e = launch_fwd(d.n, d.I, fdev, wf, f.Tf, fwd_smem_bytes(f), s);
     if (e == cudaSuccess)
         e = crowd ? launch_chain_crowd(fdev, wc, 2, crowd_smem_bytes(f), 0, s)
-                  : launch_chain(f.MN, fdev, wc, 2, chain_smem_bytes(f), cl, cthr, s);
+                  : launch_chain(f.MN, fdev, wc, 2, chain_launch_smem(f), cl, cthr, s);
     if (e == cudaSuccess) e = launch_bwd(d.n, d.I, false, fdev, wb, f.T2, bwd_smem_bytes(f, false), s);
     if (e == cudaSuccess) e = launch_finalize(fdev, wfin, nfin, 1, 0, s);
     int status = MAPDEC_OK;
