@@ -357,7 +357,8 @@ int mapdec_batch_phase_ms(mapdec_batch_t *b, double *ms);
 typedef struct {
     int P;               /* received positions per producer tile */
     int nsub;            /* producer tiles per APP super-tile */
-    int chain_budget_kb; /* shared memory of one recursion CTA, 16..220 KB */
+    int chain_budget_kb; /* shared memory of one recursion CTA, 16..220 KB (like the next
+                            field and chain_threads: of full launches' recursions) */
     int chain_stages;    /* bulk-copy stages in flight in the recursions, 2..8 */
     int store_metric;    /* 1: keep the receiver metrics R in device memory between the
                             forward and APP producers (decode only; about

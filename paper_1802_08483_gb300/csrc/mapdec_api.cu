@@ -192,10 +192,16 @@ constexpr size_t kChainSmemAlone = 200 * 1024;   // one (k_chain)
 constexpr size_t kChainSmemMost = 220 * 1024;    // beyond what an SM holds: k_chain_crowd
 constexpr int kChainMinGroups = 12;
 
-// What a frame's class asks of the recursions (0 = the planner's choice).
+// Shared memory of one recursion CTA and copy stages asked for (0 = the planner's
+// choice): of k_chain_crowd by the frame's class or the environment; of k_chain by the
+// environment alone, since classes are tuned for full launches (64 frames N = 300,
+// q = 16, n = 10, xmax = 85 with the class's 52 KB and two stages: 0.80 ms of
+// recursions, two staged chunks a step; 0.40 ms without).
 struct ChainAsk {
-    size_t budget = 0;  // shared memory of one CTA
+    size_t budget = 0;
     int stages = 0;
+    size_t chain_budget = 0;
+    int chain_stages = 0;
 };
 
 struct FrameHost {
@@ -251,12 +257,12 @@ ChainAsk chain_ask(const mapdec_tune_t *tune) {
         a.budget = (size_t)tune->chain_budget_kb * 1024;
     if (const char *e = std::getenv("MAPDEC_CHAIN_BUDGET_KB")) {  // tuning override
         const int kb = std::atoi(e);
-        if (kb >= 16 && kb <= 220) a.budget = (size_t)kb * 1024;
+        if (kb >= 16 && kb <= 220) a.budget = a.chain_budget = (size_t)kb * 1024;
     }
     if (tune && tune->chain_stages >= 2 && tune->chain_stages <= 8) a.stages = tune->chain_stages;
     if (const char *e = std::getenv("MAPDEC_CHAIN_STAGES")) {  // tuning override
         const int v = std::atoi(e);
-        if (v >= 2 && v <= 8) a.stages = v;
+        if (v >= 2 && v <= 8) a.stages = a.chain_stages = v;
     }
     return a;
 }
@@ -430,7 +436,7 @@ void plan_crowd(FrameDev &f, const ChainAsk &ask) {
 // copies in flight, row buffers, and as many copies in flight as fit (a step is
 // shorter than a copy's latency).
 void plan_chain(FrameDev &f, int cl, int threads, const ChainAsk &ask) {
-    size_t bud = ask.budget;
+    size_t bud = ask.chain_budget;
     if (bud == 0) bud = kChainSmemAlone;
     plan_crowd(f, ask);
     f.chainVC = (f.chainNV + cl - 1) / cl;
@@ -449,7 +455,7 @@ void plan_chain(FrameDev &f, int cl, int threads, const ChainAsk &ask) {
         f.chainStageFloats = (int)rup(rowsW * f.MNS + 8, 4);
         return chain_smem_bytes(f) <= budget;
     };
-    const int need = ask.stages ? ask.stages : 2;
+    const int need = ask.chain_stages ? ask.chain_stages : 2;
     // four rows are summed together, then stored one a step while the next ones
     // (and a scaled copy of the last) are written.  In a cluster two more: another
     // CTA's next row must not land where this one's storer still reads (its arrival
@@ -475,7 +481,7 @@ void plan_chain(FrameDev &f, int cl, int threads, const ChainAsk &ask) {
         }
     }
     int stages = need;
-    if (!ask.stages)
+    if (!ask.chain_stages)
         while (stages < 8 && fits(ck, stages + 1, bud)) ++stages;
     fits(ck, stages, bud);
 }
