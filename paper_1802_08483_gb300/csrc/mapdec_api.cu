@@ -1194,6 +1194,7 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
     b->d_scratch = (float *)b->dalloc(b->region_floats * 4 * b->regions + 256);
     // per-wave descriptors and work tables
     const bool segmented = b->segmented;
+    if (const char *e = std::getenv("MAPDEC_CHAIN_THREADS")) b->chain_threads = std::atoi(e);  // A/B override
     for (size_t wi = 0; wi < b->waves.size(); ++wi) {
         Wave &w = b->waves[wi];
         size_t off = (wi % b->regions) * b->region_floats;
