@@ -321,8 +321,8 @@ __device__ __forceinline__ void window_tilt(int S, int S4, int P, int BW, float 
 // A operand AB = alpha (x) beta factored, so it is never materialised.
 // smem: Rt[K][CW]  (K = P*MN, CW = NR*DS, DS = roundup4(q); column t*DS + D)
 //       Aw[P][S4], Bw[BW][S4] (BW = P + MN - 1), both carrying the tilt factors
-//       symbol constants (4 x S4), Lacc[S2][q] and Gacc[S2][3] (group = 0),
-//       Ct[3][S4][DS] (gradient)
+//       symbol constants (4 x S4), Ct[3][S4][DS] (gradient), Lacc[S2][q] and
+//       Gacc[S2][3] (group = 0)
 // ---------------------------------------------------------------------------
 template <int NB, int IB, bool GRAD>
 __global__ void __launch_bounds__(kThreads, (GRAD && (NB == 0 || NB > 10)) ? 1 : 2) k_bwd(const FrameDev *__restrict__ frames,
@@ -352,10 +352,11 @@ __global__ void __launch_bounds__(kThreads, (GRAD && (NB == 0 || NB > 10)) ? 1 :
     float *symF = reinterpret_cast<float *>(symE + Smax4);      // its fraction
     float *symG = symF + Smax4;                                 // its slope in pl
     float *symPhi = symG + Smax4;                               // theta'_{i+1} - 1
-    float *Lacc = symPhi + Smax4;
-    const bool apart = f.group != 0;  // rows of Lp and Gp per sub-tile, no accumulators
+    float *Ct = symPhi + Smax4;  // gradients
+    // accumulators, unless rows of Lp and Gp are kept per sub-tile
+    const bool apart = f.group != 0;
+    float *Lacc = GRAD ? Ct + 3 * (size_t)Smax4 * DS : Ct;
     float *Gacc = Lacc + (((size_t)f.S2 * q + 3) & ~(size_t)3);
-    float *Ct = apart ? Lacc : Gacc + (((size_t)f.S2 * 3 + 3) & ~(size_t)3);
 
     if (!apart) {
         for (int idx = threadIdx.x; idx < S2 * q; idx += blockDim.x) Lacc[idx] = 0.f;
