@@ -33,7 +33,11 @@
  *     positive sum; they are used as given (not renormalised).  NULL means
  *     uniform 1/q.
  *   - Arithmetic: FP32 for the lattice, gamma, alpha, beta and APPs; FP64 for
- *     the sum of log normalisers and for gradient reductions.
+ *     the sum of log normalisers and for gradient reductions.  Tile sizes, and
+ *     which recursion kernel runs, follow the whole batch, its memory budget and
+ *     the GPU's SM count, and with them the order of FP32 additions: a frame's
+ *     results may differ in the last bits between batches it is part of (or from
+ *     mapdec_decode's); repeated calls on one batch or handle agree bit for bit.
  *   - Every data pointer may be host or device memory (detected per call).
  *     Pinned (page-locked) host buffers of at least 1 MiB whose address is a
  *     multiple of 16 bytes are read or written by a copy kernel through their

@@ -346,7 +346,6 @@ size_t chain_smem_bytes(const FrameDev &f) {
            (size_t)f.chainStages * f.chainStageFloats * 4;
 }
 
-// MN with a compiled kernel (launches whose frames share it): n = 4 .. 12, I = 1, 2, 3.
 size_t crowd_smem_bytes(const FrameDev &f) {
     const size_t stageFloats = ((size_t)(f.crowdCD + f.MN + 1) * f.MNS + 8 + 3) & ~(size_t)3;
     return 4 * (2 * (size_t)f.Mp + (size_t)f.crowdStages * stageFloats);
@@ -367,6 +366,7 @@ cudaError_t launch_chain(int mn, const FrameDev *frames, const Work *work, int n
                          int cluster, int threads, cudaStream_t st) {
     if (nwork <= 0) return cudaSuccess;
     if (threads < 96 || threads > kChainMaxThreads || threads % 32) return cudaErrorInvalidValue;
+    // MN with a compiled kernel (launches whose frames share it): n = 4 .. 12, I = 1, 2, 3
     switch (mn) {
         case 9: case 11: case 13: case 15: case 16: case 17:
             return launch_chain_a(mn, frames, work, nwork, smem, cluster, threads, st);

@@ -18,8 +18,8 @@ constexpr int kTiltSettle = 64;  // updates every step for the first steps
 
 // ---------------------------------------------------------------------------
 // The recursions of launches with more of them than SMs (k_chain_crowd).  The same
-// recursion and the same sums in the same order as k_chain, one CTA per (frame,
-// direction), with a few registers and as little shared memory as two staged
+// recursion as k_chain, and with the default block size and chunks the same sums in
+// the same order, one CTA per (frame, direction), with a few registers and as little shared memory as two staged
 // chunks take, so that several share an SM with each other and with the producers
 // of other waves; k_chain's lower latency needs an SM to itself (256 frames N = 64,
 // q = 8: 470 us a decode with this kernel, 520 to 590 with k_chain at two and
@@ -192,7 +192,7 @@ __device__ __forceinline__ void crowd_recursion(const FrameDev &f, int tile) {
     auto issue_next = [&]() {
         const float *src = f.W + (size_t)symbol_of(is_st) * f.wblk + tab.off[is_k];
         uint64_t *b = &bar[is_slot];
-        if (!((f.test_flags & TEST_SKIP_COPY) && issued == f.test_copy)) {
+        if (!((f.test_flags & TEST_SKIP_COPY) && issued == 0)) {
             mbar_expect_tx(b, tab.bytes[is_k]);
             bulk_g2s(stage0 + (size_t)is_slot * stageFloats, src, tab.bytes[is_k], b);
         }

@@ -358,7 +358,8 @@ struct WeightTab {
 //     distributed shared memory.
 // The order of the additions is the same for every split: states are summed in
 // chunks of chainCD over 256 virtual lanes, whatever CTAs, warps and staged
-// chunks do the work; k_chain_crowd adds in that order too.
+// chunks do the work; k_chain_crowd adds in that order too with 256 threads and its
+// default chunks (another block size or budget changes its lanes per state).
 // Whole decodes with k_chain_crowd's kernel in its place and with this one: one
 // frame N = 1000, M = 401, MN = 31: 3.24 -> 1.69 ms; N = 300, M = 81, MN = 25: 638 ->
 // 420 us; gradients of N = 1000, M = 121, MN = 25: 2.36 -> 1.48 ms; 64 stream frames
@@ -369,8 +370,7 @@ struct WeightTab {
 // spill, and a cluster barrier waits for the spills' stores: 1.45 -> 1.61 ms).
 // Recursions alone, with a counter per quantity and so: N = 50, M = 41 99.9 -> 91.7
 // us; N = 300, M = 81 298 -> 282; N = 1000, M = 121 861 -> 803; N = 1000, M = 401
-// 1481 -> 1447; 64 stream frames M = 171 1141 -> 1070; against it the whole decode of
-// the 8 frames N = 8000, M = 1661 (several lane groups a warp) 198.9 -> 200.4 ms.
+// 1481 -> 1447; 64 stream frames M = 171 1141 -> 1070.
 template <int MNT, int MODE>
 __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kChainMaxThreads) k_chain(
     const FrameDev *__restrict__ frames, const Work *__restrict__ work) {
@@ -478,7 +478,8 @@ __global__ void __launch_bounds__(MODE == kChainNarrow ? kChainMostThreads : kCh
     const float *is_src = f.W + (size_t)(dir == 0 ? i0 : i1 - 1) * wblk;  // symbol block of the next copy
     const long long is_step = dir == 0 ? wblk : -wblk;
     // testing: a copy that is never issued, every CTA's first or a later one of the last CTA
-    const int skip = (f.test_flags & TEST_SKIP_COPY) && (f.test_copy == 0 || rank == ncta - 1) ? f.test_copy : -1;
+    const int tcopy = f.test_flags >> kTestCopyShift;
+    const int skip = (f.test_flags & TEST_SKIP_COPY) && (tcopy == 0 || rank == ncta - 1) ? tcopy : -1;
     auto issue_next = [&]() {
         if (lane == 0 && issued != skip) {
             const ChunkGeom g = tab[is_k];

@@ -324,11 +324,10 @@ void plan_shape(FrameDev &f, const mapdec_frame_desc_t &d, bool grad, int forceP
     f.chain_flags = 0;
     // bounded waits: a recursion gives up on a copy after this many polls
     f.wait_limit = 1u << 26;
-    f.test_flags = f.test_copy = 0;
+    f.test_flags = 0;
     if (const char *e = std::getenv("MAPDEC_TEST_STALL_CHAIN")) {  // testing: the timeout path
         if (std::atoi(e) >= 1) {
-            f.test_flags |= TEST_SKIP_COPY;
-            f.test_copy = std::atoi(e) - 1;
+            f.test_flags = TEST_SKIP_COPY | (std::atoi(e) - 1) << kTestCopyShift;
             f.wait_limit = 4096;
         }
     }
@@ -562,6 +561,8 @@ bool plan_bwd_tc(FrameDev &f) {
 
 // Tiles with rows of APP partial sums of their own, and their positions.
 size_t row_tiles(const FrameDev &f) { return f.group ? f.T : f.T2; }
+// CTAs of the APP producer in a gradient call.
+int grad_tiles(const FrameDev &f) { return f.ps ? f.T2 : (f.T + f.gsub - 1) / f.gsub; }
 long long row_positions(const FrameDev &f) { return (long long)f.P * (f.group ? 1 : f.nsub); }
 
 size_t frame_scratch_floats(const FrameDev &f, bool grad) {
@@ -674,6 +675,7 @@ void fill_tiles(FrameHost &h, long long pos, long long ctas, bool grad, bool fil
     if (fill && h.fit && h.split) fit_app_tile(f, pos);
     if (h.fit && !h.tc && (fill || !h.store)) fit_fwd_tile(f, pos, grad);
     if (fill && h.split) split_supertiles(f, supertile_split(ctas));
+    f.gsub = f.nsub;
     if (fill && h.rows) {
         // eight CTAs per SM, no more sub-tiles each than planned; the order of the sums
         // stays that of the planned super-tiles.  A launch that has as many CTAs with
@@ -683,8 +685,9 @@ void fill_tiles(FrameHost &h, long long pos, long long ctas, bool grad, bool fil
         if (nsub == 1 || nsub < f.nsub) {
             f.group = f.nsub;
             f.S2 = f.S;
-            f.nsub = nsub;
-            f.T2 = (f.T + nsub - 1) / nsub;
+            f.gsub = nsub;
+            f.nsub = 1;
+            f.T2 = f.T;
         }
     }
 }
@@ -713,6 +716,7 @@ struct ClassLaunch {
     bool ps = false;   // per-symbol-codebook producers (producers_ps.cuh)
     Work *d_fwd = nullptr; int nfwd = 0; size_t smem_fwd = 0;
     Work *d_bwd = nullptr; int nbwd = 0; size_t smem_bwd = 0;
+    Work *d_bwdg = nullptr; int nbwdg = 0;  // the APP producer's in gradient calls
 };
 
 // One segment index of a segmented wave: descriptors and work lists.
@@ -906,7 +910,7 @@ void build_segments(mapdec_batch *b, Wave &w, const std::vector<FrameDev> &devs,
             c.tc = (std::get<2>(kv.first) & kTcFwd) != 0;
             c.tcb = (std::get<2>(kv.first) & kTcBwd) != 0;
             c.ps = (std::get<2>(kv.first) & kPerSym) != 0;
-            std::vector<Work> fw, bwk;
+            std::vector<Work> fw, bwk, bwg;
             for (int k : kv.second) {
                 const FrameHost &h = b->fr[w.f0 + k];
                 if (s >= h.nseg) continue;
@@ -916,6 +920,8 @@ void build_segments(mapdec_batch *b, Wave &w, const std::vector<FrameDev> &devs,
                 const long long phi = std::min(f.rho, (long long)f.n * (f.seg_i1 - 1) + f.xmax);
                 for (long long t = plo / f.Pf; t <= phi / f.Pf; ++t) fw.push_back({k, (int)t});
                 for (long long t = plo / P2; t <= phi / P2; ++t) bwk.push_back({k, (int)t});
+                const long long Pg = (long long)f.P * f.gsub;
+                for (long long t = plo / Pg; t <= phi / Pg; ++t) bwg.push_back({k, (int)t});
                 c.smem_fwd = std::max(c.smem_fwd, c.tc ? fwd_tc_smem_bytes(f) : fwd_smem_bytes(f));
                 c.smem_bwd = std::max(c.smem_bwd, c.ps    ? bwd_ps_smem_bytes(f, b->grad)
                                                   : c.tcb ? bwd_tc_smem_bytes(f)
@@ -923,6 +929,7 @@ void build_segments(mapdec_batch *b, Wave &w, const std::vector<FrameDev> &devs,
             }
             upload(fw, c.d_fwd, c.nfwd);
             upload(bwk, c.d_bwd, c.nbwd);
+            if (b->grad) upload(bwg, c.d_bwdg, c.nbwdg);
             sl.cls.push_back(c);
         }
     }
@@ -1345,11 +1352,12 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
             c.tc = (std::get<2>(kv.first) & kTcFwd) != 0;
             c.tcb = (std::get<2>(kv.first) & kTcBwd) != 0;
             c.ps = (std::get<2>(kv.first) & kPerSym) != 0;
-            std::vector<Work> fw, bw;
+            std::vector<Work> fw, bw, bwg;
             for (int k : kv.second) {
                 const FrameDev &f = devs[k];
                 for (int t = 0; t < f.Tf; ++t) fw.push_back({k, t});
                 for (int t = 0; t < f.T2; ++t) bw.push_back({k, t});
+                for (int t = 0; t < grad_tiles(f); ++t) bwg.push_back({k, t});
                 c.smem_fwd = std::max(c.smem_fwd, c.tc ? fwd_tc_smem_bytes(f) : fwd_smem_bytes(f));
                 c.smem_bwd = std::max(c.smem_bwd, c.ps    ? bwd_ps_smem_bytes(f, b->grad)
                                                   : c.tcb ? bwd_tc_smem_bytes(f)
@@ -1361,6 +1369,11 @@ int build_batch(mapdec_batch *b, const mapdec_frame_desc_t *frames, int nf, int 
             c.d_bwd = (Work *)b->dalloc(sizeof(Work) * bw.size());
             CK(cudaMemcpy(c.d_fwd, fw.data(), sizeof(Work) * fw.size(), cudaMemcpyHostToDevice));
             CK(cudaMemcpy(c.d_bwd, bw.data(), sizeof(Work) * bw.size(), cudaMemcpyHostToDevice));
+            if (b->grad) {
+                c.nbwdg = (int)bwg.size();
+                c.d_bwdg = (Work *)b->dalloc(sizeof(Work) * bwg.size());
+                CK(cudaMemcpy(c.d_bwdg, bwg.data(), sizeof(Work) * bwg.size(), cudaMemcpyHostToDevice));
+            }
             w.cls.push_back(c);
         }
         if (segmented) build_segments(b, w, devs, byclass);
@@ -1464,9 +1477,11 @@ int64_t enqueue_run(mapdec_batch *b, bool grad, cudaStream_t st) {
         CK(cudaStreamWaitEvent(st, b->dep[2 * w + 1], 0));
         mark(w, 3, 0, st);
         for (auto &c : wv.cls) {
-            CK(c.ps    ? launch_bwd_ps(c.n, c.I, grad, wv.d_frames, c.d_bwd, c.nbwd, c.smem_bwd, st)
-               : c.tcb ? launch_bwd_tc(c.n, c.I, wv.d_frames, c.d_bwd, c.nbwd, c.smem_bwd, st)
-                       : launch_bwd(c.n, c.I, grad, wv.d_frames, c.d_bwd, c.nbwd, c.smem_bwd, st));
+            const Work *bw = grad ? c.d_bwdg : c.d_bwd;
+            const int nbw = grad ? c.nbwdg : c.nbwd;
+            CK(c.ps    ? launch_bwd_ps(c.n, c.I, grad, wv.d_frames, bw, nbw, c.smem_bwd, st)
+               : c.tcb ? launch_bwd_tc(c.n, c.I, wv.d_frames, bw, nbw, c.smem_bwd, st)
+                       : launch_bwd(c.n, c.I, grad, wv.d_frames, bw, nbw, c.smem_bwd, st));
             ++launches;
         }
         mark(w, 3, 1, st);
@@ -1569,7 +1584,8 @@ int64_t enqueue_run_seg(mapdec_batch *b, bool grad, cudaStream_t st) {
             for (auto &c : sl.cls) {
                 if (c.nbwd == 0) continue;
                 CK(c.tcb ? launch_bwd_tc(c.n, c.I, sl.d_frames, c.d_bwd, c.nbwd, c.smem_bwd, st)
-                         : launch_bwd(c.n, c.I, grad, sl.d_frames, c.d_bwd, c.nbwd, c.smem_bwd, st));
+                         : launch_bwd(c.n, c.I, grad, sl.d_frames, grad ? c.d_bwdg : c.d_bwd,
+                                      grad ? c.nbwdg : c.nbwd, c.smem_bwd, st));
                 ++launches;
             }
             CK(launch_finalize(sl.d_frames, sl.d_fin, sl.nfin, nw, grad ? 1 : 0, st,
@@ -2116,6 +2132,7 @@ void retarget_single(mapdec_batch *b, int64_t rho, bool ext, const float *phi0,
     for (auto &c : w.cls) {
         c.nfwd = f.Tf;
         c.nbwd = f.T2;
+        c.nbwdg = grad_tiles(f);
     }
     CK(cudaMemcpyAsync(w.d_frames, &f, sizeof(FrameDev), cudaMemcpyHostToDevice, b->stream));
 }

@@ -18,7 +18,8 @@ constexpr int CH_SEGMENTED = 1;   // start/end rows and controller state come fr
 constexpr int CH_REPLAY = 2;      // forward chain replays the recorded tilts (recompute sweep)
 
 // test_flags
-constexpr int TEST_SKIP_COPY = 1;  // one of a recursion's copies is never issued
+constexpr int TEST_SKIP_COPY = 1;  // one of a recursion's copies is never issued ..
+constexpr int kTestCopyShift = 1;  // .. number test_flags >> 1 (k_chain_crowd: the first)
 
 constexpr int kMaxI = 7;        // insertion cap supported by the kernels
 constexpr int kMaxMN = 64;      // n(I+1) + 1 <= 64 (received window fits 64 bits)
@@ -83,8 +84,7 @@ struct FrameDev {
     int chainVWarps;  // virtual warps with lanes (<= 8)
     int chainWarps, chainList;  // compute warps of the launch, lane groups of one (and an end mark)
     uint32_t wait_limit;  // polls before a recursion's wait on a copy gives up (ST_TIMEOUT)
-    int test_flags;       // TEST_SKIP_COPY: copy number test_copy is never issued (tests the timeout path)
-    int test_copy;
+    int test_flags;       // TEST_SKIP_COPY (tests the timeout path)
     long long rho;
     long long wblk;  // floats per symbol block of W (M * MNS rounded up to 4)
     // FP32 lattice constants.  Every received bit carries a weight kappa: the
@@ -134,6 +134,11 @@ struct FrameDev {
     double *loglik;  // 1
     double *dchan;   // 3 or null
     int *status;     // 1
+    // Sub-tiles per CTA in gradient calls: nsub, but with group > 0 (a decode's CTA then
+    // takes one, nsub = 1) as many as fill the GPU.  Last, where it moves no field that
+    // k_chain_crowd reads at every step: among the producers' fields 512 mixed frames
+    // took 164.4 ms, here 162.9, and 256 frames of N = 64 471 us, here 466.
+    int gsub;
 };
 
 constexpr int kChainRowPad = 96;  // zeros on both sides of a row (k_chain reads the band past it)
@@ -173,10 +178,10 @@ __host__ __device__ inline void tile_symbols(const FrameDev &f, int tile, int &i
     const long long p0 = (long long)tile * f.Pf;
     range_symbols(f, p0, p0 + f.Pf - 1, ilo, ihi);
 }
-// Backward super-tile t covers positions [t P nsub, (t+1) P nsub - 1].
-__host__ __device__ inline void super_symbols(const FrameDev &f, int tile, int &ilo, int &ihi) {
-    const long long p0 = (long long)tile * f.P * f.nsub;
-    range_symbols(f, p0, p0 + (long long)f.P * f.nsub - 1, ilo, ihi);
+// Backward super-tile t of nsub sub-tiles covers positions [t P nsub, (t+1) P nsub - 1].
+__host__ __device__ inline void super_symbols(const FrameDev &f, int nsub, int tile, int &ilo, int &ihi) {
+    const long long p0 = (long long)tile * f.P * nsub;
+    range_symbols(f, p0, p0 + (long long)f.P * nsub - 1, ilo, ihi);
 }
 
 // 64 received bits starting at position p: bit k = y_{k+1} = Y[p + k].

@@ -82,15 +82,16 @@ cudaError_t launch_pack(const FrameDev *frames, const uint8_t *const *rx_bytes,
                         uint32_t *const *rx_words, int nframes, long long max_words,
                         cudaStream_t st);
 size_t chain_smem_bytes(const FrameDev &f);
-// cluster: CTAs per recursion (1, 2, 4 or 8); threads: a multiple of 32 from 96 to
-// 512 (the last two warps move data, the others compute; one CTA of more than
-// 320: a warp per lane group instead of one per virtual warp)
 // Recursions of launches with more of them than SMs; threads 128, 256 or 512
 // (anything else: 256).
 size_t crowd_smem_bytes(const FrameDev &f);
 cudaError_t launch_chain_crowd(const FrameDev *frames, const Work *work, int nwork, size_t smem,
                                int threads, cudaStream_t st);
-// mn: the frames' common MN, 0 where they differ (or always: the general kernel)
+// mn: the frames' common MN, 0 where they differ (or always: the general kernel);
+// smem: the larger of chain_smem_bytes and crowd_smem_bytes; cluster: CTAs per
+// recursion (1, 2, 4 or 8); threads: a multiple of 32 from 96 to 512 (the last two
+// warps move data, the others compute; one CTA of more than 320: a warp per lane
+// group instead of one per virtual warp)
 cudaError_t launch_chain(int mn, const FrameDev *frames, const Work *work, int nwork, size_t smem,
                          int cluster, int threads, cudaStream_t st);
 #define MAPDEC_DECLARE_CHAIN(G)                                                              \

@@ -43,8 +43,8 @@ __device__ __forceinline__ void lattice_any(const FrameDev &f, uint32_t x, uint6
 // select per value took up to a tenth of a lattice's instructions; 64 stream frames
 // N = 1000, q = 16, n = 10: k_fwd 1092 -> 1053 us, k_bwd 1265 -> 1232 us; 48 gradient
 // frames N = 2000, q = 32, n = 8, whole pass 35.5 -> 34.3 ms; 16 frames N = 150,
-// n = 15 892 -> 864 us; 8 frames N = 8000, n = 12, I = 3 200.4 -> 200.7 ms, where the
-// values' count is large and the branch gives nothing).
+// n = 15 892 -> 864 us; against it 8 frames N = 8000, n = 12, I = 3, where the values
+// are many, 198.8 -> 200.4 ms).
 // MODE 0 -> R; MODE k > 0 -> the k-th tangent.
 template <int NB, int IB, int MODE>
 __device__ __forceinline__ void eval_metric(const FrameDev &f, long long p, int D, float *out) {
@@ -308,9 +308,9 @@ __device__ __forceinline__ void window_tilt(int S, int S4, int P, int BW, float 
 // Backward producer (APP partial sums, optional tangents).  One CTA owns a
 // super-tile of nsub sub-tiles of P positions and accumulates, in shared
 // memory, for every symbol i it touches (gradient frames of launches that planned
-// super-tiles cannot fill, f.group > 0, in decode calls too: stores for every
-// sub-tile, so that the CTAs can be short enough to fill the GPU while finalize adds
-// the sub-tiles up in one fixed order; 48 frames N = 2000, q = 32, segments of 45
+// super-tiles cannot fill, f.group > 0: keeps the sums of every sub-tile, so that the
+// CTAs can be short enough to fill the GPU while finalize adds the sub-tiles up in
+// one fixed order; 48 frames N = 2000, q = 32, segments of 45
 // symbols: super-tiles of 42 sub-tiles were 144 CTAs a launch, the whole pass
 // 67.4 ms; of 3 sub-tiles 41.3 ms):
 //   Lacc[i][D] = sum_{p in super-tile, j} alpha_i(s') R[p][D][j] beta_{i+1}(s'+j-n)
@@ -335,7 +335,7 @@ __global__ void __launch_bounds__(kThreads, (GRAD && (NB == 0 || NB > 10)) ? 1 :
     const int q = f.q, P = f.P;
     const long long rho = f.rho;
     int ilo2, ihi2;
-    super_symbols(f, wk.tile, ilo2, ihi2);
+    super_symbols(f, GRAD ? f.gsub : f.nsub, wk.tile, ilo2, ihi2);
     const int S2 = ihi2 - ilo2 + 1;
     if (S2 <= 0) return;
     const int DS = (q + 3) & ~3;
@@ -353,8 +353,10 @@ __global__ void __launch_bounds__(kThreads, (GRAD && (NB == 0 || NB > 10)) ? 1 :
     float *symG = symF + Smax4;                                 // its slope in pl
     float *symPhi = symG + Smax4;                               // theta'_{i+1} - 1
     float *Ct = symPhi + Smax4;  // gradients
-    // accumulators, unless rows of Lp and Gp are kept per sub-tile
-    const bool apart = f.group != 0;
+    // Rows of Lp and Gp per sub-tile are stored as they are formed.  A decode of such a
+    // frame has one sub-tile per CTA, and nothing to tell apart (with a test in its inner
+    // loops 512 mixed frames took 165.4 ms, without 162.5).
+    const bool apart = GRAD && f.group != 0;
     float *Lacc = GRAD ? Ct + 3 * (size_t)Smax4 * DS : Ct;
     float *Gacc = Lacc + (((size_t)f.S2 * q + 3) & ~(size_t)3);
 
@@ -364,8 +366,8 @@ __global__ void __launch_bounds__(kThreads, (GRAD && (NB == 0 || NB > 10)) ? 1 :
             for (int idx = threadIdx.x; idx < S2 * 3; idx += blockDim.x) Gacc[idx] = 0.f;
     }
 
-    for (int sub = 0; sub < f.nsub; ++sub) {
-        const long long p0 = ((long long)wk.tile * f.nsub + sub) * P;
+    for (int sub = 0; sub < (GRAD ? f.gsub : f.nsub); ++sub) {
+        const long long p0 = ((long long)wk.tile * (GRAD ? f.gsub : f.nsub) + sub) * P;
         if (p0 > rho) break;
         int ilo, ihi;
         range_symbols(f, p0, p0 + P - 1, ilo, ihi);
@@ -374,7 +376,7 @@ __global__ void __launch_bounds__(kThreads, (GRAD && (NB == 0 || NB > 10)) ? 1 :
         const int S4 = (S + 3) & ~3;
         const int off = ilo - ilo2;  // row of symbol ilo in the accumulators
         // the sub-tile's rows of Lp and Gp
-        const size_t row0 = (size_t)((long long)wk.tile * f.nsub + sub) * f.S2;
+        const size_t row0 = (size_t)((long long)wk.tile * f.gsub + sub) * f.S2;
 
         // (B) alpha and beta windows of the sub-tile's symbols (see
         // window_constants / window_fetch); the raw rows land while the

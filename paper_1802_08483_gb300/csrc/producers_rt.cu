@@ -33,7 +33,8 @@ size_t bwd_smem_bytes(const FrameDev &f, bool grad) {
     if (grad) fl += 3 * Smax4 * DS;
     // the accumulators: none with rows per sub-tile, but tiles are planned with room
     // for them (the tiles fix the order of the gradient's sums)
-    if (f.group == 0)
+    // (a decode's for its one sub-tile take the place of the staged tangent sums)
+    if (!grad || f.group == 0)
         fl += (((size_t)f.S2 * f.q + 3) & ~(size_t)3) + (((size_t)f.S2 * 3 + 3) & ~(size_t)3);
     return 4 * fl;
 }

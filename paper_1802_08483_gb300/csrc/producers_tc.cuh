@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_tc(const FrameDev *__restri
     const int q = f.q, P = f.P;
     const long long rho = f.rho;
     int ilo2, ihi2;
-    super_symbols(f, wk.tile, ilo2, ihi2);
+    super_symbols(f, f.nsub, wk.tile, ilo2, ihi2);
     const int S2 = ihi2 - ilo2 + 1;
     if (S2 <= 0) return;  // uniform over the CTA, before any tensor memory is held
     const int Kp = (P * MNp + 15) & ~15;
