@@ -255,7 +255,7 @@ def run_oracle(frames_idx, cores):
 
 
 PHASE_KERNELS = {"pack": "k_pack", "forward": "k_fwd, all (n, I) classes",
-                 "chains": "k_chain", "backward": "k_bwd, all (n, I) classes",
+                 "chains": "k_chain_crowd, k_chain", "backward": "k_bwd, all (n, I) classes",
                  "finalize": "k_finalize"}
 
 
